@@ -93,63 +93,6 @@ namespace {
 __constant__ float c_fz[FzTab<3>::SIZE];
 }
 
-// Exact zeros of the 1D tables: a Gauss rule with an odd number of points
-// has a node at 0, where the odd Legendre polynomials and the derivatives of
-// the even ones vanish, and Pt_0' = 0 everywhere. The multiply-adds by them
-// are dropped at compile time (the loops are unrolled); for finite operands
-// the sums are unchanged, bit for bit.
-template <int K>
-__host__ __device__ constexpr bool zero_p(int u, int q) {
-  return K % 2 == 0 && 2 * q == K && u % 2 == 1;
-}
-template <int K>
-__host__ __device__ constexpr bool zero_d(int u, int q) {
-  return u == 0 || (K % 2 == 0 && 2 * q == K && u % 2 == 0);
-}
-
-// mode index of the exponents along (normal, tangential 1, tangential 2) of a
-// face normal to axis D (tangential axes in ascending order)
-template <int D>
-__host__ __device__ constexpr int face_mode(int e, int a, int b) {
-  return D == 0 ? mode_index(e, a, b) : (D == 1 ? mode_index(a, e, b) : mode_index(a, b, e));
-}
-
-// an upper bound of |x| in binary32 from the high word of x (20 fraction
-// bits, rounded up: at most 2^-20 above |x|); magnitudes below 2^-126 map to
-// 2^-126, huge and non-finite values to infinity
-__device__ __forceinline__ float abs_up(double x) {
-  unsigned u = (unsigned)__double2hiint(x) & 0x7fffffffu;
-  u = min(max(u, 0x38100000u), 0x47efffffu);
-  return __uint_as_float(((u - 0x38000000u) << 3) + 8u);
-}
-
-// binary64 -> binary32 on the integer pipe (no FP64-unit conversion):
-// rounded to nearest on the 29 dropped fraction bits (ties away from zero,
-// which differs from ties-to-even only when they are exactly 2^28);
-// magnitudes below 2^-126 give a signed zero, magnitudes of 2^128 and above,
-// infinities and NaNs a signed infinity (the stage's screen then queues the
-// cell and the full limiter reports the non-finite state)
-__device__ __forceinline__ float f64_to_f32_q(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned mag = hi & 0x7fffffffu;
-  unsigned r = (__funnelshift_l(lo, hi, 3) - 0xC0000000u) + ((lo >> 28) & 1u);
-  r = mag < 0x38100000u ? 0u : r;
-  r = mag >= 0x47f00000u ? 0x7f800000u : r;
-  return __uint_as_float(r | (hi & 0x80000000u));
-}
-
-// binary32 -> binary64 on the integer pipe: exact for normal numbers,
-// subnormals give a signed zero, infinities and NaNs stay what they are
-__device__ __forceinline__ double f32_to_f64_q(float x) {
-  const unsigned u = __float_as_uint(x), mag = u & 0x7fffffffu, sg = u & 0x80000000u;
-  unsigned hi = sg | ((mag >> 3) + 0x38000000u);
-  unsigned lo = u << 29;
-  hi = mag >= 0x7f800000u ? (hi | 0x7ff00000u) : hi;
-  hi = mag < 0x00800000u ? sg : hi;
-  lo = mag < 0x00800000u ? 0u : lo;
-  return __hiloint2double((int)hi, (int)lo);
-}
-
 __device__ __forceinline__ void prefetch_l1(const void* p) {
 #ifdef __CUDA_ARCH__
   asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
@@ -166,26 +109,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 #endif
 }
 
-// approximate reciprocal and reciprocal square root (one MUFU operation
-// each, subnormals flushed to zero: relative error of a few ulp)
-__device__ __forceinline__ float rcp_fast(float x) {
-#ifdef __CUDA_ARCH__
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-#else
-  return 1.f / x;
-#endif
-}
-__device__ __forceinline__ float rsqrt_fast(float x) {
-#ifdef __CUDA_ARCH__
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-#else
-  return 1.f / std::sqrt(x);
-#endif
-}
 // sqrt(max(x, 0)): 0 for x <= 0, the limit of a sound speed at p -> 0+
 __device__ __forceinline__ float sqrt_fast(float x) { return x > 0.f ? x * rsqrt_fast(x) : 0.f; }
 
@@ -367,39 +290,6 @@ __device__ __forceinline__ void fz_apply(const float (&Hl)[(K + 1) * (K + 2) / 2
         acc[m] = fmaf(c_fz[TB::EM + e], Hl[j], acc[m]);
         acc[m] = fmaf(-c_fz[TB::EP + e], Hh[j], acc[m]);
       }
-}
-
-// position of conserved variable i in the frame of a face normal to axis d:
-// (rho, m_n, m_t1, m_t2, E) with t1 < t2 the other two axes. Traces and
-// fluxes are stored in this order, so the numerical flux is evaluated with
-// a compile-time normal and no reordering.
-__device__ __forceinline__ int face_var(int d, int i) {
-  if (i == 0 || i == 4) return i;
-  const int ax = i - 1, t1 = d == 0 ? 1 : 0;
-  return ax == d ? 1 : (ax == t1 ? 2 : 3);
-}
-
-// Sufficient limiter screen in FP32 from the cell means m and the excursion
-// bounds s_i >= sum_{l>=1} |w_il| max|phi_l|: true when the density and the
-// pressure provably stay above the floors at every point of the limiter's
-// point set (same bounds as the FP64 screen, multiplied through by the
-// density bound, with a 1e-5 relative margin that covers the FP32 rounding
-// of the inputs and of the test). NaN inputs fail.
-__device__ __forceinline__ bool screen_f32(const float* m, const float* s, float gm1, float er, float ep) {
-  const float r = m[0];
-  const float rlo = r - s[0];
-  if (!(rlo >= er + 1e-5f * (fabsf(r) + s[0]))) return false;
-  float k2 = 0.f;
-#pragma unroll
-  for (int a = 1; a <= 3; ++a) {
-    const float mh = fabsf(m[a]) + s[a];
-    k2 = fmaf(mh, mh, k2);
-  }
-  k2 *= 0.5f;
-  const float elo = m[4] - s[4];
-  const float lhs = gm1 * fmaf(elo, rlo, -k2);
-  const float rhs = fmaf(ep, rlo, 1e-5f * gm1 * fmaf(fabsf(m[4]) + s[4], rlo, k2));
-  return lhs >= rhs;
 }
 
 template <int K, bool FORCE, int FLUX>

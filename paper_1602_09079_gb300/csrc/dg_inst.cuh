@@ -40,10 +40,11 @@ const float* tab_ptr<float>() { return h_tab32[cur_dev()]; }
 
 inline unsigned grid1(long long n, int per) { return (unsigned)((n + per - 1) / per); }
 
-// FP32 degrees 0-2: tiled register kernels; sum factorisation pays from
-// degree 2 on (fewer multiply-adds than the dense quadrature)
+// FP32 degrees 0-2: tiled register kernels, degree 3 sum-factorised; FP64:
+// the fixed-point sum-factorised kernel from degree 1 on (at degree 0 there is
+// one point and nothing to factorise)
 constexpr bool kRegF32 = KK <= 2;
-constexpr bool kSumFact = KK >= 2;
+constexpr bool kSumFact = KK >= 1;
 
 template <typename T, int MODE, bool FORCE>
 cudaError_t set_volume_smem() {
@@ -84,10 +85,10 @@ cudaError_t upload(const double* h64, const float* h32) {
     for (int i = 0; i < NSF; ++i) f32[i] = (float)f64[i];
     if ((e = cudaMemcpyToSymbol(c_sf64, f64, sizeof(double) * NSF)) != cudaSuccess) return e;
     if ((e = cudaMemcpyToSymbol(c_sf32, f32, sizeof(float) * NSF)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(face_sf64_kernel<KK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(face_sf64_kernel<KK, 0, kSumFact>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)FaceSF64<KK>::smem())) != cudaSuccess)
       return e;
-    if ((e = cudaFuncSetAttribute(face_sf64_kernel<KK, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(face_sf64_kernel<KK, 1, kSumFact>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)FaceSF64<KK>::smem())) != cudaSuccess)
       return e;
   }
@@ -114,19 +115,28 @@ cudaError_t upload(const double* h64, const float* h32) {
     for (cudaError_t x : f)
       if (x != cudaSuccess) r = x;
   }
-  cudaError_t s[8] = {set_volume_smem<double, MODE_RHS, false>(),  set_volume_smem<double, MODE_RHS, true>(),
-                      set_volume_smem<double, MODE_STAGE, false>(), set_volume_smem<double, MODE_STAGE, true>(),
-                      set_volume_smem<float, MODE_RHS, false>(),   set_volume_smem<float, MODE_RHS, true>(),
-                      set_volume_smem<float, MODE_STAGE, false>(),  set_volume_smem<float, MODE_STAGE, true>()};
+  cudaError_t s[4] = {set_volume_smem<double, MODE_RHS, false>(), set_volume_smem<double, MODE_RHS, true>(),
+                      set_volume_smem<double, MODE_STAGE, false>(), set_volume_smem<double, MODE_STAGE, true>()};
   for (cudaError_t x : s)
     if (x != cudaSuccess) r = x;
+  if constexpr (!kRegF32) {
+    cudaError_t f[4] = {set_volume_smem<float, MODE_RHS, false>(), set_volume_smem<float, MODE_RHS, true>(),
+                        set_volume_smem<float, MODE_STAGE, false>(), set_volume_smem<float, MODE_STAGE, true>()};
+    for (cudaError_t x : f)
+      if (x != cudaSuccess) r = x;
+  }
   return r;
 }
 
 template <int FLUX>
 cudaError_t face64(const double* y, void* fh, const Geo& g, Ctrl* ctrl, cudaStream_t s) {
   using CF = FaceSF64<KK>;
-  face_sf64_kernel<KK, FLUX><<<grid1(g.nc, 32), CF::THREADS, CF::smem(), s>>>(y, static_cast<double*>(fh), g, ctrl);
+  // one direction per CTA while the tiles alone fill less than half of the
+  // chip's CTA slots (6 x 8 x 7 at degree 2: 21 us instead of 52; from there on
+  // the second load of a tile's coefficients costs what the waves gain)
+  const unsigned tiles = grid1(g.nc, 32);
+  face_sf64_kernel<KK, FLUX, kSumFact><<<dim3(tiles, tiles * 2 < 152u * CF::MINB ? 3 : 1), CF::THREADS, CF::smem(), s>>>(
+      y, static_cast<double*>(fh), g, ctrl);
   return cudaGetLastError();
 }
 
@@ -185,8 +195,7 @@ cudaError_t volume_rhs(int prec, bool force, const double* y, const float* yf, c
     if (prec)
       return force ? vol_f32<MODE_RHS, true>(yf, fh, field, g, st, R, ctrl, s)
                    : vol_f32<MODE_RHS, false>(yf, fh, field, g, st, R, ctrl, s);
-  }
-  if (prec)
+  } else if (prec)
     return force ? vol_t<float, MODE_RHS, true>(y, yf, fh, field, g, st, R, ctrl, s)
                  : vol_t<float, MODE_RHS, false>(y, yf, fh, field, g, st, R, ctrl, s);
   return force ? vol_t<double, MODE_RHS, true>(y, yf, fh, field, g, st, R, ctrl, s)
@@ -201,8 +210,7 @@ cudaError_t volume_stage(int prec, bool force, const void* fh, const void* field
     if (prec)
       return force ? vol_f32<MODE_STAGE, true>(yf, fh, field, g, st, nullptr, ctrl, s)
                    : vol_f32<MODE_STAGE, false>(yf, fh, field, g, st, nullptr, ctrl, s);
-  }
-  if (prec)
+  } else if (prec)
     return force ? vol_t<float, MODE_STAGE, true>(ys, yf, fh, field, g, st, nullptr, ctrl, s)
                  : vol_t<float, MODE_STAGE, false>(ys, yf, fh, field, g, st, nullptr, ctrl, s);
   return force ? vol_t<double, MODE_STAGE, true>(ys, yf, fh, field, g, st, nullptr, ctrl, s)

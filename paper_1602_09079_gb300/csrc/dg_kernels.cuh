@@ -17,7 +17,9 @@
 
 namespace dg {
 
-constexpr int kThreads = 256;
+// threads per CTA of the tiled kernels: a multiple of the 5 (k + 1) (cell,
+// variable, slice) roles per cell of volume_sf_kernel at every degree
+constexpr int kThreads = 240;
 
 enum VolMode { MODE_RHS = 0, MODE_STAGE = 1 };
 
@@ -325,112 +327,195 @@ __device__ __forceinline__ unsigned face_f32_dir(const float* __restrict__ yf, f
   return err;
 }
 
-// Face fluxes, FP64, sum-factorised traces: tile of 32 cells, warp d = face
-// direction (the low face of each cell). Both cells' coefficients are
-// contracted along the normal with Pt_e(+-1) into the tangential
-// coefficients E[i][(a,b)]; then, per tangential Gauss row t2,
-// H[i][a] = sum_b E[i][(a,b)] Pt_b(t2) and per point U_i = sum_a H[i][a]
-// Pt_a(t1) (E and H in shared memory, one column per thread): 5 (Q T + Q^2 (k+1))
-// multiply-adds per side instead of 5 N Q^2.
+// Face fluxes, FP64: tile of 32 cells, one direction after the other. One
+// (cell, variable) per thread (warp = variable) contracts the coefficients of
+// its cell and of the lower neighbour along the normal with Pt_e(-+1) into the
+// tangential coefficients E, then along t2 and t1 to the values at the face's
+// Q^2 points, all in 64-bit fixed point (dg_common.cuh): both sides' values go
+// to shared memory in the face's frame. Then one numerical flux per face point
+// in FP64, which is what bounds the kernel (27 HLLC fluxes of about 105 FP64
+// operations per cell at degree 2, 2 operations per clock and SM). The fluxes go
+// out as their T = (K+1)(K+2)/2 moments with the tangential modes,
+// [3][5][T][n_cells], once for the two cells that need them (MOMENTS; for the
+// dense volume_kernel the fluxes at the points, [3][5][Q^2][n_cells]). With FP64 contractions
+// and the 190-operation HLLC the kernel took 21.2 ms at 128^3, degree 2, now
+// 11.1 (the FP64 operations alone: 9.3).
 template <int K>
 struct FaceSF64 {
-  static constexpr int TP = (K + 1) * (K + 2) / 2;
-  static constexpr int THREADS = 96;
-  // per thread: E of both sides (2 x 5 x TP) and H of both sides (2 x 5 x (K+1))
-  static constexpr size_t smem() { return sizeof(double) * 2 * 5 * (TP + K + 1) * THREADS; }
+  static constexpr int C = 32, THREADS = 5 * C;
+  static constexpr int Q2 = (K + 1) * (K + 1), T = (K + 1) * (K + 2) / 2;
+  // 4 CTAs per SM (96 registers) keep the FP64 pipe busier than 3 without
+  // spills: 11.1 against 12.6 ms at 128^3, degree 2
+  static constexpr int MINB = 4;
+  // values [side][variable][point][cell]
+  static constexpr size_t smem() { return sizeof(double) * 2 * 5 * Q2 * C; }
 };
 
-template <int K, int D, int FLUX>
-__device__ __forceinline__ unsigned face_sf64_dir(const double* __restrict__ y, double* __restrict__ fh,
-                                                  const Geo& g, long long c, int ix, int iy, int iz, double* sE) {
-  constexpr int N = nmodes(K), Q = K + 1, KP = K + 1, Q2 = Q * Q, TP = FaceSF64<K>::TP;
-  constexpr int TH = FaceSF64<K>::THREADS, FE = 3 * KP * Q;
-  const long long nc = g.nc;
-  const long long cl = neighbour(g, ix, iy, iz, D, -1);
-  double* eL = sE + threadIdx.x;                  // [i][pair] column of this thread
-  double* eR = sE + 5 * TP * TH + threadIdx.x;
+// coefficients of one (cell, variable) in fixed point, exponent B; row stride nc
+template <int K>
+__device__ __forceinline__ void fx_load(const double* __restrict__ p, size_t nc, Fx (&x)[nmodes(K)], int& B) {
+  constexpr int N = nmodes(K);
+  double w[N];
 #pragma unroll
-  for (int j = 0; j < 5 * TP; ++j) {
-    eL[j * TH] = 0.0;
-    eR[j * TH] = 0.0;
-  }
-  // one mode at a time (few live registers): its exponent along the normal
-  // selects Pt_e(+-1), the tangential pair selects the E entry
-#pragma unroll 1
-  for (int m = 0; m < N; ++m) {
-    int u, v, w;
-    mode_uvw(m, u, v, w);
-    const int e = D == 0 ? u : (D == 1 ? v : w);
-    const int j = pair_index(K, D == 0 ? v : u, D == 2 ? v : w);
-    const double pl = c_sf64[FE + KP + e];  // lower cell, xi_d = +1
-    const double pr = c_sf64[FE + e];       // own cell, xi_d = -1
+  for (int l = 0; l < N; ++l) w[l] = __ldg(p + (size_t)l * nc);
+  B = fx_bound<K>(w);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      eL[(i * TP + j) * TH] += __ldg(y + (size_t)(i * N + m) * nc + cl) * pl;
-      eR[(i * TP + j) * TH] += __ldg(y + (size_t)(i * N + m) * nc + c) * pr;
-    }
-  }
-  const double gamma = g.gamma;
-  unsigned err = 0;
-  double* hLp = sE + 2 * 5 * TP * TH + threadIdx.x;  // [i][a] column of this thread
-  double* hRp = hLp + 5 * KP * TH;
-#pragma unroll 1
-  for (int t2 = 0; t2 < Q; ++t2) {
-#pragma unroll 1
-    for (int i = 0; i < 5; ++i)
-#pragma unroll
-      for (int a = 0; a <= K; ++a) {
-        double sl = 0.0, sr = 0.0;
-#pragma unroll
-        for (int b = 0; a + b <= K; ++b) {
-          const double pb = c_sf64[b * Q + t2];
-          const int j = pair_index(K, a, b);
-          sl += eL[(i * TP + j) * TH] * pb;
-          sr += eR[(i * TP + j) * TH] * pb;
-        }
-        hLp[(i * KP + a) * TH] = sl;
-        hRp[(i * KP + a) * TH] = sr;
-      }
-#pragma unroll 1
-    for (int t1 = 0; t1 < Q; ++t1) {
-      double UL[5], UR[5];
-#pragma unroll
-      for (int i = 0; i < 5; ++i) {
-        double ul = 0.0, ur = 0.0;
-#pragma unroll
-        for (int a = 0; a <= K; ++a) {
-          const double pa = c_sf64[a * Q + t1];
-          ul += hLp[(i * KP + a) * TH] * pa;
-          ur += hRp[(i * KP + a) * TH] * pa;
-        }
-        UL[i] = ul;
-        UR[i] = ur;
-      }
-      double F[5];
-      err |= riemann_flux<FLUX, double>(D, UL, UR, gamma, F);
-      const int p = t1 + Q * t2;
-#pragma unroll
-      for (int i = 0; i < 5; ++i) fh[((size_t)(D * 5 + i) * Q2 + p) * nc + c] = F[i];
-    }
-  }
-  return err;
+  for (int l = 0; l < N; ++l) x[l] = fx_split(fx_from(w[l], B));
 }
 
-template <int K, int FLUX>
-__global__ void __launch_bounds__(FaceSF64<K>::THREADS) face_sf64_kernel(const double* __restrict__ y,
+// rows of a triangle E[(a, b)] at the nodes along b: H[q][a] = sum_b E[(a, b)] Pt_b(q)
+template <int K, int A>
+__device__ __forceinline__ void fx_rows(const Fx (&E)[(K + 1) * (K + 2) / 2], Fx (&H)[K + 1][K + 1]) {
+  if constexpr (A <= K) {
+    Fx e[K + 1 - A];
+    long long v[K + 1];
+#pragma unroll
+    for (int b = 0; b + A <= K; ++b) e[b] = E[pair_index(K, A, b)];
+    fx_values<K, K + 1 - A>(e, v);
+#pragma unroll
+    for (int q = 0; q <= K; ++q) H[q][A] = fx_split(v[q]);
+    fx_rows<K, A + 1>(E, H);
+  }
+}
+
+// values on face (D, S) (S = 0: xi_D = -1, S = 1: xi_D = +1) at the points
+// t1 + Q t2, rows of 32 cells apart
+template <int K, int D, int S>
+__device__ __forceinline__ void fx_trace(const Fx (&x)[nmodes(K)], int B, double* dst) {
+  using FT = FxTab<K>;
+  constexpr int Q = K + 1, T = (K + 1) * (K + 2) / 2;
+  const double bad = __longlong_as_double(0x7ff8000000000000LL);
+  Fx E[T];
+#pragma unroll
+  for (int a = 0, j = 0; a <= K; ++a)
+#pragma unroll
+    for (int b = 0; a + b <= K; ++b, ++j) {
+      FxAcc s{0, 0};
+#pragma unroll
+      for (int e = 1; e + a + b <= K; ++e) fx_madt(s, x[face_mode<D>(e, a, b)], FT::E + S * (K + 1) + e);
+      // Pt_0 = 1
+      E[j] = fx_split(fx_val(s) + fx_join(x[face_mode<D>(0, a, b)]));
+    }
+  Fx H[Q][K + 1];  // [t2][a]
+  fx_rows<K, 0>(E, H);
+#pragma unroll
+  for (int t2 = 0; t2 < Q; ++t2) {
+    long long v[Q];
+    fx_values<K, K + 1>(H[t2], v);
+#pragma unroll
+    for (int t1 = 0; t1 < Q; ++t1) dst[(t1 + Q * t2) * 32] = B < kFxHuge ? fx_to_double(v[t1], B) : bad;
+  }
+}
+
+// T moments sum_{t1,t2} F(t1 + Q t2) P'_a(t1) P'_b(t2), P' = Pt w / 2, of the
+// flux values f (Q^2 rows of 32 cells), to m (rows nc apart)
+template <int K>
+__device__ __forceinline__ void fx_moments(const double* f, double* __restrict__ m, size_t nc) {
+  constexpr int Q = K + 1, Q2 = Q * Q;
+  unsigned mx = 0;
+#pragma unroll
+  for (int p = 0; p < Q2; ++p) mx = max(mx, (unsigned)__double2hiint(f[p * 32]) & 0x7fffffffu);
+  const int B = max(kFxTiny, bexp(mx) + 1);
+  const double bad = __longlong_as_double(0x7ff8000000000000LL);
+  long long G[K + 1][Q];  // [a][t2]
+#pragma unroll
+  for (int t2 = 0; t2 < Q; ++t2) {
+    long long v[Q];
+#pragma unroll
+    for (int t1 = 0; t1 < Q; ++t1) v[t1] = fx_from(f[(t1 + Q * t2) * 32], B);
+    FxAcc g[K + 1];
+#pragma unroll
+    for (int a = 0; a <= K; ++a) g[a] = {0, 0};
+    fx_project<K, false>(v, g);
+#pragma unroll
+    for (int a = 0; a <= K; ++a) G[a][t2] = fx_val(g[a]);
+  }
+#pragma unroll
+  for (int a = 0, j = 0; a <= K; ++a) {
+    FxAcc h[K + 1];
+#pragma unroll
+    for (int b = 0; b <= K; ++b) h[b] = {0, 0};
+    fx_project<K, false>(G[a], h);
+#pragma unroll
+    for (int b = 0; a + b <= K; ++b, ++j) m[(size_t)j * nc] = B < kFxHuge ? fx_to_double(fx_val(h[b]), B) : bad;
+  }
+}
+
+template <int K, int FLUX, bool MOMENTS = (K >= 2)>
+__global__ void __launch_bounds__(FaceSF64<K>::THREADS, FaceSF64<K>::MINB) face_sf64_kernel(const double* __restrict__ y,
                                                                          double* __restrict__ fh, Geo g, Ctrl* ctrl) {
+  using CF = FaceSF64<K>;
+  constexpr int N = nmodes(K), C = CF::C, Q2 = CF::Q2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* sE = reinterpret_cast<double*>(smem_raw);
-  const long long c = (long long)blockIdx.x * 32 + (threadIdx.x & 31);
-  if (c >= g.nc) return;  // no block-wide barrier below
-  const int d = threadIdx.x >> 5;  // warp-uniform direction
-  int ix, iy, iz;
-  cell_xyz(c, g, ix, iy, iz);
-  unsigned e;
-  if (d == 0) e = face_sf64_dir<K, 0, FLUX>(y, fh, g, c, ix, iy, iz, sE);
-  else if (d == 1) e = face_sf64_dir<K, 1, FLUX>(y, fh, g, c, ix, iy, iz, sE);
-  else e = face_sf64_dir<K, 2, FLUX>(y, fh, g, c, ix, iy, iz, sE);
-  if (e) atomicOr(&ctrl->err, e);
+  double* sU = reinterpret_cast<double*>(smem_raw);
+  const long long nc = g.nc, c0 = (long long)blockIdx.x * C;
+  const int c = threadIdx.x % C, i = threadIdx.x / C;  // i: conserved variable, warp-uniform
+  const long long cell = c0 + c;
+  const bool live = cell < nc;
+  int ix = 0, iy = 0, iz = 0;
+  Fx x[N];
+  int B = 0;
+  const double* yi = y + (size_t)(i * N) * nc;
+  if (live) {
+    cell_xyz(cell, g, ix, iy, iz);
+    fx_load<K>(yi + cell, nc, x, B);
+  }
+  unsigned err = 0;
+  // directions blockIdx.y, + gridDim.y, ...: all in one CTA, or one per CTA
+  // where a mesh has too few tiles to fill the chip
+#pragma unroll 1
+  for (int d = blockIdx.y; d < 3; d += gridDim.y) {
+    if (live) {
+      // row of this variable in the face's frame (rho, m_n, m_t1, m_t2, E)
+      double* dst = sU + face_var(d, i) * Q2 * C + c;
+      Fx xl[N];
+      int Bl;
+      fx_load<K>(yi + neighbour(g, ix, iy, iz, d, -1), nc, xl, Bl);
+      if (d == 0) {
+        fx_trace<K, 0, 1>(xl, Bl, dst);
+        fx_trace<K, 0, 0>(x, B, dst + 5 * Q2 * C);
+      } else if (d == 1) {
+        fx_trace<K, 1, 1>(xl, Bl, dst);
+        fx_trace<K, 1, 0>(x, B, dst + 5 * Q2 * C);
+      } else {
+        fx_trace<K, 2, 1>(xl, Bl, dst);
+        fx_trace<K, 2, 0>(x, B, dst + 5 * Q2 * C);
+      }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int it = threadIdx.x; it < Q2 * C; it += CF::THREADS) {
+      const int p = it / C, cc = it % C;
+      if (c0 + cc < nc) {
+        double UL[5], UR[5], F[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          UL[v] = sU[(v * Q2 + p) * C + cc];
+          UR[v] = sU[((5 + v) * Q2 + p) * C + cc];
+        }
+        if constexpr (FLUX == 1) err |= exact_flux<double>(0, UL, UR, g.gamma, F);
+        else hllc64_x(UL, UR, g.gamma, F);
+        // the flux takes the left values' place (or goes out as it is)
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          if constexpr (MOMENTS) {
+            sU[(v * Q2 + p) * C + cc] = F[v];
+          } else {
+            // position of the frame's component v among (rho, m_x, m_y, m_z, E)
+            const int ax = v == 1 ? d : (v == 2 ? (d == 0 ? 1 : 0) : (d == 2 ? 1 : 2));
+            fh[((size_t)(d * 5 + ((v == 0 || v == 4) ? v : 1 + ax)) * Q2 + p) * nc + c0 + cc] = F[v];
+          }
+        }
+      }
+    }
+    if constexpr (MOMENTS) {
+      __syncthreads();
+      if (live)
+        fx_moments<K>(sU + face_var(d, i) * Q2 * C + c, fh + (size_t)(d * 5 + i) * CF::T * nc + cell, nc);
+    }
+    __syncthreads();
+  }
+  if (err) atomicOr(&ctrl->err, err);
 }
 
 // CTAs per SM the face kernel's register budget is sized for (measured at
@@ -794,20 +879,10 @@ __global__ void __launch_bounds__(kThreads) screen_kernel(const double* __restri
 }
 
 // ============================================== sum-factorised volume kernel
-// FP64 path (and the FP32 path of degree 3): the tensor-product structure of
-// the complete-degree basis turns each contraction over the Q^3 points into
-// three one-dimensional ones (sum factorisation), every stage a cooperative
-// pass of the block over (cell, index) items in shared memory:
-//  values   A1[u,v][c] = sum_w w_uvw P_w(c); A2[u][b,c] = sum_v A1[u,v][c] P_v(b);
-//           U[a,b,c] = sum_u A2[u][b,c] P_u(a)
-//  fluxes   G_d = F_d(U) / (4 dx_d) at every point (and S/8 for the source)
-//  project  H_d[u][b,c] = sum_a G_d X_d(u,a); J[u,v][c] = sum_b H_0 Pw + H_1 Dw;
-//           I2[u,v][c] = sum_b H_2 Pw; dw_uvw = sum_c J Pw(w,c) + I2 Dw(w,c)
-//           (X_0 = Dw, X_1 = X_2 = Pw; Pw = P w_a, Dw = P' w_a)
-//  faces    Mt[a][t2] = sum_t1 Fhat Pw(a,t1); M[a,b] = +-sum_t2 Mt Pw(b,t2)/(4 dx_d);
-//           expanded along the normal by Pt_e(-1) (low face) or Pt_e(+1) (high).
-// Multiply-adds per cell and variable at degree 2: 165 for the values, 465
-// for the projection, 55 per face (dense quadrature: 270, 810, 90).
+// The tensor-product structure of the complete-degree basis turns each
+// contraction over the Q^3 points into three one-dimensional ones (sum
+// factorisation). Multiply-adds per cell and variable at degree 2: 165 for the
+// values, 465 for the projection, 55 per face (dense quadrature: 270, 810, 90).
 template <int K, typename T>
 struct VolSF {
   static constexpr int Q = K + 1, KP = K + 1, Q2 = Q * Q, Q3 = Q * Q * Q, N = nmodes(K), TP = (K + 1) * (K + 2) / 2;
@@ -816,10 +891,22 @@ struct VolSF {
   // buffer 1: A1, U, H, M; buffer 2: A2, fluxes, (J, I2, SI | Mt)
   static constexpr int BUF1 = mx(mx(5 * TP * Q, 5 * Q3), mx(19 * KP * Q2, 30 * TP));
   static constexpr int BUF2 = mx(mx(5 * KP * Q2, 19 * Q3), MT0 + 30 * KP * Q);
-  static constexpr int C = sizeof(T) == 8 ? (K >= 3 ? 4 : 8) : 8;
-  static constexpr size_t smem() {
-    return (size_t)C * (8 * (5 * N + 10) + sizeof(T) * (BUF1 + BUF2));
-  }
+  static constexpr int C = 8;
+  static constexpr size_t smem() { return (size_t)C * (8 * (5 * N + 10) + sizeof(T) * (BUF1 + BUF2)); }
+};
+// FP64: one (cell, variable, slice of constant z) per thread
+template <int K>
+struct VolSF<K, double> {
+  static constexpr int Q = K + 1, Q3 = Q * Q * Q, N = nmodes(K);
+  static constexpr int C = kThreads / (5 * Q);
+  // shared memory in doubles: values [5][Q3][C], fluxes and sources [13][Q3][C];
+  // then, over both, the slices' sums [Q][5 N][C] (64-bit integers), their
+  // exponents [Q][5][C] (int), and the screen's [Q + 1][5][C] (float)
+  static constexpr int U = 0, F = 5 * Q3 * C, EXPS = Q * 5 * N * C, SCREEN = EXPS + (Q * 5 * C + 1) / 2;
+  static constexpr int A = 18 * Q3 * C, B = SCREEN + ((Q + 1) * 5 * C + 1) / 2, END = A > B ? A : B;
+  static constexpr size_t smem() { return sizeof(double) * END; }
+  // CTAs per SM the register budget is sized for (128 registers)
+  static constexpr int MINB = 2;
 };
 
 template <int K>
@@ -833,250 +920,385 @@ __device__ __forceinline__ void pair_uv(int j, int& u, int& v) {
 }
 
 
-// Cooperative form (FP64): one output per (cell, index) item, inner loops
-// over the exact triangular ranges, so no FP64 multiply-add is issued for an
-// absent mode (the FP64 pipe is the bound).
+// raises the accumulators' exponent A to B (never lowers it)
+template <int N>
+__device__ __forceinline__ void fx_raise(long long (&acc)[N], int& A, int B) {
+  if (B > A) {
+    const int d = min(B - A, 63);
+#pragma unroll
+    for (int m = 0; m < N; ++m) acc[m] >>= d;
+    A = B;
+  }
+}
+
+// acc += the two faces normal to D, from the moments of their fluxes (low face
+// at ml, high face at mh, rows nc apart; face_sf64_kernel): Pt_e(-1) M_low -
+// Pt_e(+1) M_high for the mode e along D, Pt_e(-1) = (-1)^e Pt_e(+1); the
+// moments times inv_dx[D] 2^-p = S 2^-58 (unity: 1)
+template <int K, int D>
+__device__ __forceinline__ void fx_apply(const long long (&even)[(K + 1) * (K + 2) / 2],
+                                         const long long (&odd)[(K + 1) * (K + 2) / 2],
+                                         long long (&acc)[nmodes(K)]) {
+  constexpr int F = FxTab<K>::F + K + 1;
+#pragma unroll
+  for (int a = 0, j = 0; a <= K; ++a)
+#pragma unroll
+    for (int b = 0; a + b <= K; ++b, ++j) {
+      acc[face_mode<D>(0, a, b)] += even[j] >> 4;  // Pt_0 / 16
+      const Fx ev = fx_split(even[j]), od = fx_split(odd[j]);
+#pragma unroll
+      for (int e = 1; e + a + b <= K; ++e) {
+        FxAcc t{0, 0};
+        fx_madt(t, e % 2 ? od : ev, F + e);
+        acc[face_mode<D>(e, a, b)] += e % 2 ? -fx_val(t) : fx_val(t);
+      }
+    }
+}
+__device__ __forceinline__ long long fx_scaled(long long x, bool unity, Fx S) {
+  if (unity) return x;
+  FxAcc t{0, 0};
+  fx_mad(t, fx_split(x), S.h, S.l);
+  return fx_val(t);
+}
+template <int K>
+__device__ __forceinline__ void fx_faces(int d, const double* __restrict__ ml, const double* __restrict__ mh,
+                                         size_t nc, bool unity, Fx S, long long (&acc)[nmodes(K)], int& A, int& top) {
+  constexpr int T = (K + 1) * (K + 2) / 2;
+  double l[T], h[T];
+  unsigned mx = 0;
+#pragma unroll
+  for (int j = 0; j < T; ++j) {
+    l[j] = __ldg(ml + (size_t)j * nc);
+    h[j] = __ldg(mh + (size_t)j * nc);
+    mx = max(mx, max((unsigned)__double2hiint(l[j]) & 0x7fffffffu, (unsigned)__double2hiint(h[j]) & 0x7fffffffu));
+  }
+  top = max(top, bexp(mx));
+  fx_raise(acc, A, bexp(mx) + 1);
+  long long even[T], odd[T];
+#pragma unroll
+  for (int j = 0; j < T; ++j) {
+    const long long a = fx_scaled(fx_from(l[j], A), unity, S), b = fx_scaled(fx_from(h[j], A), unity, S);
+    even[j] = a - b;
+    odd[j] = a + b;
+  }
+  if (d == 0) fx_apply<K, 0>(even, odd, acc);
+  else if (d == 1) fx_apply<K, 1>(even, odd, acc);
+  else fx_apply<K, 2>(even, odd, acc);
+}
+
+// Volume integral, surface integral and stage update, FP64. One (cell,
+// variable, slice of constant z) per thread for the contractions, which run in
+// 64-bit fixed point (dg_common.cuh) with one exponent per variable's
+// coefficients and one, raised as the terms come, for the thread's sums of
+// dw/dt (its slice, and the faces of the directions z, z + Q, ...); one (cell,
+// point) per thread for the Euler fluxes and the driving source, in FP64; then
+// one (cell, variable) and every Q-th mode per thread for the sum over the
+// slices and the stage update. Everything enters the sums as
+//   dw/dt = 2^(p + 4) [sum_d s_d sum_q F_d(q) (D'/8) P' P' + sum_faces +- s_d
+//           (P' P' moments) Pt_e / 16 + sum_q 2^-(p+4) S(q) P' P' P'],
+// P' = P w / 2 and D' = (dP/dxi) w / 2 (sums of |P'| <= 1, of |D'| / 8 <= 0.61),
+// 2^p >= 1/dx_d = s_d 2^p. Inputs take 60 bits and the source 58, so that no
+// intermediate reaches 2^61 and no sum 2^63. Integer issue bounds it on large
+// meshes (128^3, degree 2: 7.7 ms per stage, the FP64 contractions took 33.6;
+// 64^3, degree 3: 2.2 ms) and one thread's chain on small ones, which is why a
+// slice is a thread's work: with a thread per (cell, variable) 128^3 took 7.1
+// ms, but 8 x 8 x 8 at degree 1 or 33 x 32 x 31 fill the chip with three or
+// four times the threads (8^3: 11 us, the dense kernel took 84).
 template <int K, typename T, int MODE, bool FORCE>
-__global__ void __launch_bounds__(kThreads) volume_sf_kernel(const double* __restrict__ yin,
-                                                             const float* __restrict__ yf32, const T* __restrict__ fh,
-                                                             const T* __restrict__ field, const T* __restrict__ tab,
-                                                             const double* __restrict__ tab64, Geo g, StageArgs st,
-                                                             double* __restrict__ R, Ctrl* ctrl) {
+__global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
+    volume_sf_kernel(const double* __restrict__ yin, const float* __restrict__ yf32, const T* __restrict__ fh,
+                     const T* __restrict__ field, const T* __restrict__ tab, const double* __restrict__ tab64, Geo g,
+                     StageArgs st, double* __restrict__ R, Ctrl* ctrl) {
+  static_assert(sizeof(T) == 8, "fixed-point form: FP64 path only");
   using TB = Tab<K>;
-  using CF = VolSF<K, T>;
-  constexpr int N = TB::N, Q = CF::Q, Q2 = CF::Q2, Q3 = CF::Q3, TP = CF::TP, C = CF::C, KP = K + 1;
+  using CF = VolSF<K, double>;
+  using FT = FxTab<K>;
+  constexpr int N = TB::N, Q = K + 1, Q2 = Q * Q, Q3 = TB::Q3, C = CF::C, T2 = (K + 1) * (K + 2) / 2;
+  static_assert(kThreads == 5 * Q * C, "one (cell, variable, slice) per thread");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double* sV = reinterpret_cast<double*>(smem_raw);  // stage output (FP64)
-  double* sM = sV + 5 * N * C;
-  double* sA = sM + 5 * C;
-  T* sW = reinterpret_cast<T*>(sV);  // stage input (T), read only by the first pass
-  T* b1 = reinterpret_cast<T*>(sA + 5 * C);
-  T* b2 = b1 + CF::BUF1 * C;
+  double* sm64 = reinterpret_cast<double*>(smem_raw);
   const long long nc = g.nc;
   const long long c0 = (long long)blockIdx.x * C;
   const int tid = threadIdx.x;
-  const T* P1 = tab + TB::P1;
-  const T* P1W = tab + TB::P1W;
-  const T* D1W = tab + TB::D1W;
-  // stage input: FP64 state (T = double) or its FP32 shadow (T = float)
+  const int c = tid % C, i = (tid / C) % 5, qz = tid / (5 * C);
+  const long long cell = c0 + c;
+  const bool live = cell < nc;
+  const long long cellc = live ? cell : nc - 1;  // ragged tail: in-bounds reads, nothing written
   const double* ysrc = (MODE == MODE_STAGE) ? st.ys : yin;
-  const float* yfsrc = (MODE == MODE_STAGE) ? st.yf : yf32;
-  for (int it = tid; it < 5 * N * C; it += kThreads) {
-    const int c = it % C, r = it / C;
-    const long long cell = c0 + c;
-    T v = r == 0 ? T(1) : T(0);
-    if (cell < nc) {
-      if constexpr (sizeof(T) == 4) v = yfsrc[(size_t)r * nc + cell];
-      else v = ysrc[(size_t)r * nc + cell];
+  int top = 0;  // largest exponent seen
+  // --------------------------------------------- values at the slice's points
+  {
+    Fx x[N];
+    int B;
+    fx_load<K>(ysrc + (size_t)(i * N) * nc + cellc, nc, x, B);
+    if (B >= kFxHuge) top = kFxHuge;
+    Fx pz[K + 1];  // Pt_w at the slice
+#pragma unroll
+    for (int ww = 1; ww <= K; ++ww) pz[ww] = {c_fx[FT::P + ww * Q + qz][0], c_fx[FT::P + ww * Q + qz][1]};
+    Fx A1[T2];
+#pragma unroll
+    for (int u = 0, j = 0; u <= K; ++u)
+#pragma unroll
+      for (int v = 0; u + v <= K; ++v, ++j) {
+        FxAcc s{0, 0};
+#pragma unroll
+        for (int ww = 1; u + v + ww <= K; ++ww) fx_mad(s, x[mode_index(u, v, ww)], pz[ww].h, pz[ww].l);
+        const long long x0 = fx_join(x[mode_index(u, v, 0)]);
+        A1[j] = fx_split(u + v < K ? fx_val(s) + x0 : x0);
+      }
+    Fx A2[Q][K + 1];  // [qy][u]
+    fx_rows<K, 0>(A1, A2);
+    double* u = sm64 + CF::U + (i * Q3 + qz * Q2) * C + c;
+#pragma unroll
+    for (int qy = 0; qy < Q; ++qy) {
+      long long v[Q];
+      fx_values<K, K + 1>(A2[qy], v);
+#pragma unroll
+      for (int qx = 0; qx < Q; ++qx) u[(qx + Q * qy) * C] = fx_to_double(v[qx], B);
     }
-    sW[r * C + c] = v;
   }
-  __syncthreads();
-  // A1[i][pair(u,v)][qc] -> b1
-  for (int it = tid; it < 5 * TP * Q * C; it += kThreads) {
-    const int c = it % C, r = it / C, qc = r % Q, j = (r / Q) % TP, i = r / (Q * TP);
-    int u, v;
-    pair_uv<K>(j, u, v);
-    T a = T(0);
-    for (int w = 0; w <= K - u - v; ++w) a += sW[(i * N + mode_index(u, v, w)) * C + c] * __ldg(P1 + w * Q + qc);
-    b1[it] = a;
-  }
-  __syncthreads();
-  // A2[i][u][qb + Q qc] -> b2
-  for (int it = tid; it < 5 * KP * Q2 * C; it += kThreads) {
-    const int c = it % C, r = it / C, bc = r % Q2, u = (r / Q2) % KP, i = r / (Q2 * KP);
-    const int qb = bc % Q, qc = bc / Q;
-    T a = T(0);
-    for (int v = 0; v <= K - u; ++v) a += b1[((i * TP + pair_index(K, u, v)) * Q + qc) * C + c] * __ldg(P1 + v * Q + qb);
-    b2[it] = a;
-  }
-  __syncthreads();
-  // U[i][qa + Q qb + Q2 qc] -> b1
-  for (int it = tid; it < 5 * Q3 * C; it += kThreads) {
-    const int c = it % C, r = it / C, q = r % Q3, i = r / Q3;
-    const int qa = q % Q, bc = q / Q;
-    T a = T(0);
+  // 2^p >= every 1/dx; s_d = 1/dx_d 2^-p as a multiplier S 2^-58 (1: skipped)
+  const double im = fmax(g.inv_dx[0], fmax(g.inv_dx[1], g.inv_dx[2]));
+  const int pb = bexp((unsigned)__double2hiint(im)) + ((__double_as_longlong(im) & 0xfffffffffffffLL) ? 1 : 0);
+  const int p4 = pb - 1023 + 4;
+  const double unit = __hiloint2double(pb << 20, 0);
+  long long acc[N];
 #pragma unroll
-    for (int u = 0; u <= K; ++u) a += b2[((i * KP + u) * Q2 + bc) * C + c] * __ldg(P1 + u * Q + qa);
-    b1[it] = a;
+  for (int l = 0; l < N; ++l) acc[l] = 0;
+  int A = kFxTiny;
+  {
+    int ix, iy, iz;
+    cell_xyz(cellc, g, ix, iy, iz);
+#pragma unroll 1
+    for (int d = qz; d < 3; d += Q) {
+      const double* f = fh + (size_t)((d * 5 + i) * T2) * nc;
+      const double idx = d == 0 ? g.inv_dx[0] : (d == 1 ? g.inv_dx[1] : g.inv_dx[2]);
+      fx_faces<K>(d, f + cellc, f + neighbour(g, ix, iy, iz, d, 1), nc, idx == unit, fx_split(fx_from(idx, pb) >> 2),
+                  acc, A, top);
+    }
   }
   __syncthreads();
-  // fluxes G[d*5+i][q] = F_d / (4 dx_d), source S[i-1][q] = S / 8 -> b2
-  const T gm1 = (T)(g.gamma - 1.0);
-  for (int it = tid; it < Q3 * C; it += kThreads) {
-    const int c = it % C, q = it / C;
-    T U[5];
+  // ------------------------------ Euler fluxes and the driving source, FP64
+  const double gm1 = g.gamma - 1.0;
+  {
+    const double* sU = sm64 + CF::U;
+    double* sF = sm64 + CF::F;
+    constexpr int R3 = Q3 * C;
+#pragma unroll 1
+    for (int it = tid; it < R3; it += kThreads) {
+      double a[3];
+      if (FORCE) {
+        const int q = it / C, cc = it % C;
+        const T* ap = field + (size_t)q * nc + (c0 + cc < nc ? c0 + cc : nc - 1);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) U[i] = b1[(i * Q3 + q) * C + c];
-    const T ir = T(1) / U[0];
-    const T v[3] = {U[1] * ir, U[2] * ir, U[3] * ir};
-    const T p = gm1 * (U[4] - T(0.5) * U[0] * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]));
+        for (int d = 0; d < 3; ++d) a[d] = __ldg(ap + (size_t)d * Q3 * nc);
+      }
+      const double r = sU[it], m0 = sU[R3 + it], m1 = sU[2 * R3 + it], m2 = sU[3 * R3 + it], E = sU[4 * R3 + it];
+      const double ir = rcp64(r);
+      const double v0 = m0 * ir, v1 = m1 * ir, v2 = m2 * ir;
+      const double p = gm1 * fma(-0.5, fma(m0, v0, fma(m1, v1, m2 * v2)), E);
+      const double h = E + p;
+      sF[it] = fma(m0, v0, p);
+      sF[R3 + it] = m0 * v1;
+      sF[2 * R3 + it] = m0 * v2;
+      sF[3 * R3 + it] = fma(m1, v1, p);
+      sF[4 * R3 + it] = m1 * v2;
+      sF[5 * R3 + it] = fma(m2, v2, p);
+      sF[6 * R3 + it] = h * v0;
+      sF[7 * R3 + it] = h * v1;
+      sF[8 * R3 + it] = h * v2;
+      if (FORCE) {
+        sF[9 * R3 + it] = r * a[0];
+        sF[10 * R3 + it] = r * a[1];
+        sF[11 * R3 + it] = r * a[2];
+        sF[12 * R3 + it] = fma(m0, a[0], fma(m1, a[1], m2 * a[2]));
+      }
+    }
+  }
+  __syncthreads();
+  // -------------------- projection onto the basis gradients (and the source)
+  {
+    // where this variable's fluxes along x, y, z and its source lie: the mass
+    // flux is the momentum itself, the momentum flux is symmetric
+    const int sym[3] = {i == 1 ? 0 : i == 2 ? 1 : 2, i == 1 ? 1 : i == 2 ? 3 : 4, i == 1 ? 2 : i == 2 ? 4 : 5};
+    const double* fd[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      fd[d] = (i == 0 ? sm64 + CF::U + (1 + d) * Q3 * C : sm64 + CF::F + (i == 4 ? 6 + d : sym[d]) * Q3 * C) +
+              qz * Q2 * C + c;
+    const double* fs = sm64 + CF::F + ((9 + (i > 0 ? i - 1 : 0)) * Q3 + qz * Q2) * C + c;
+    const bool src = FORCE && i > 0;
+    bool one[3];
+    Fx S[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      T F[5];
-      euler_flux<T>(d, U, v, p, F);
-      const T sc = (T)(0.25 * g.inv_dx[d]);
-#pragma unroll
-      for (int i = 0; i < 5; ++i) b2[((d * 5 + i) * Q3 + q) * C + c] = F[i] * sc;
+      one[d] = g.inv_dx[d] == unit;
+      S[d] = fx_split(fx_from(g.inv_dx[d], pb) >> 2);
     }
-    if (FORCE) {
-      const long long cell = c0 + c < nc ? c0 + c : nc - 1;  // ragged tail: in-bounds reads
-      T a[3];
+    unsigned mx = 0, ms = 0;
 #pragma unroll
-      for (int d = 0; d < 3; ++d) a[d] = __ldg(field + ((size_t)d * Q3 + q) * nc + cell);
-      const T e8 = T(0.125);
-      b2[((15 + 0) * Q3 + q) * C + c] = U[0] * a[0] * e8;
-      b2[((15 + 1) * Q3 + q) * C + c] = U[0] * a[1] * e8;
-      b2[((15 + 2) * Q3 + q) * C + c] = U[0] * a[2] * e8;
-      b2[((15 + 3) * Q3 + q) * C + c] = (U[1] * a[0] + U[2] * a[1] + U[3] * a[2]) * e8;
-    }
-  }
-  __syncthreads();
-  // H[comp][u][qb + Q qc] = sum_a G[comp][qa,qb,qc] X(u,qa) -> b1
-  constexpr int NCP = FORCE ? 19 : 15;
-  for (int it = tid; it < NCP * KP * Q2 * C; it += kThreads) {
-    const int c = it % C, r = it / C, bc = r % Q2, u = (r / Q2) % KP, comp = r / (Q2 * KP);
-    const T* X = (comp < 5) ? D1W : P1W;
-    T a = T(0);
+      for (int q = 0; q < Q2; ++q) {
 #pragma unroll
-    for (int qa = 0; qa < Q; ++qa) a += b2[(comp * Q3 + qa + Q * bc) * C + c] * __ldg(X + u * Q + qa);
-    b1[it] = a;
-  }
-  __syncthreads();
-  // rows 0..4: J_i = sum_b H_{0,i} Pw + H_{1,i} Dw; rows 5..9: I2_i = sum_b H_{2,i} Pw;
-  // rows 10..13: SI = sum_b SH Pw -> b2[row][pair][qc]. Face moments
-  // Mt[d*2+side][i][a][t2] = sum_t1 Fhat Pw(a, t1) -> b2 + MT0
-  constexpr int NR = FORCE ? 14 : 10;
-  constexpr int NJ = NR * TP * Q * C;
-  for (int it = tid; it < NJ + 30 * Q * C; it += kThreads) {
-    if (it < NJ) {
-      const int c = it % C, r = it / C, qc = r % Q, j = (r / Q) % TP, row = r / (Q * TP);
-      int u, v;
-      pair_uv<K>(j, u, v);
-      T a = T(0);
-      if (row < 5) {
-        const T* h0 = b1 + ((row * KP + u) * Q2) * C;
-        const T* h1 = b1 + (((5 + row) * KP + u) * Q2) * C;
-#pragma unroll
-        for (int qb = 0; qb < Q; ++qb)
-          a += h0[(qb + Q * qc) * C + c] * __ldg(P1W + v * Q + qb) + h1[(qb + Q * qc) * C + c] * __ldg(D1W + v * Q + qb);
-      } else {
-        const int comp = row < 10 ? 10 + (row - 5) : 15 + (row - 10);
-        const T* h = b1 + ((comp * KP + u) * Q2) * C;
-#pragma unroll
-        for (int qb = 0; qb < Q; ++qb) a += h[(qb + Q * qc) * C + c] * __ldg(P1W + v * Q + qb);
+        for (int d = 0; d < 3; ++d) mx = max(mx, (unsigned)__double2hiint(fd[d][q * C]) & 0x7fffffffu);
+        if (src) ms = max(ms, (unsigned)__double2hiint(fs[q * C]) & 0x7fffffffu);
       }
-      b2[it] = a;
-    } else {
-      const int jt = it - NJ;
-      const int c = jt % C, r = jt / C, t2 = r % Q, i = (r / Q) % 5, ds = r / (5 * Q);
-      const int d = ds >> 1, side = ds & 1;
-      const long long cell = c0 + c;
-      T m[KP];
+      top = max(top, max(bexp(mx), bexp(ms)));
+      fx_raise(acc, A, max(bexp(mx) + 1, ms ? bexp(ms) - p4 + 3 : 0));
+      // rows of constant y: Gx, Gy, Gz = sums along x
+      auto row = [&](int qy, long long (&gx)[K + 1], long long (&gy)[K + 1], long long (&gz)[K + 1]) {
+        FxAcc G[K + 1];
+        long long f[Q];
 #pragma unroll
-      for (int a = 0; a <= K; ++a) m[a] = T(0);
-      if (cell < nc) {
-        long long fc = cell;  // low face: this cell's; high face: the upper cell's
-        if (side) {
-          int ix, iy, iz;
-          cell_xyz(cell, g, ix, iy, iz);
-          fc = neighbour(g, ix, iy, iz, d, +1);
+        for (int u = 0; u <= K; ++u) G[u] = {0, 0};
+#pragma unroll
+        for (int q = 0; q < Q; ++q) f[q] = fx_scaled(fx_from(fd[0][(q + Q * qy) * C], A), one[0], S[0]);
+        fx_project<K, true>(f, G);
+        if (src) {
+          // weighted by P' along all three axes, like the x flux along y and
+          // z: it joins the x flux's sums here
+#pragma unroll
+          for (int q = 0; q < Q; ++q) f[q] = fx_from(fs[(q + Q * qy) * C], A + p4);
+          fx_project<K, false>(f, G);
         }
-        const T* fp = fh + ((size_t)(d * 5 + i) * Q2 + Q * t2) * nc + fc;
 #pragma unroll
-        for (int t1 = 0; t1 < Q; ++t1) {
-          const T f = __ldg(fp + (size_t)t1 * nc);
+        for (int u = 0; u <= K; ++u) {
+          gx[u] = fx_val(G[u]);
+          G[u] = {0, 0};
+        }
 #pragma unroll
-          for (int a = 0; a <= K; ++a) m[a] += f * __ldg(P1W + a * Q + t1);
+        for (int q = 0; q < Q; ++q) f[q] = fx_scaled(fx_from(fd[1][(q + Q * qy) * C], A), one[1], S[1]);
+        fx_project<K, false>(f, G);
+#pragma unroll
+        for (int u = 0; u <= K; ++u) {
+          gy[u] = fx_val(G[u]);
+          G[u] = {0, 0};
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) f[q] = fx_scaled(fx_from(fd[2][(q + Q * qy) * C], A), one[2], S[2]);
+        fx_project<K, false>(f, G);
+#pragma unroll
+        for (int u = 0; u <= K; ++u) gz[u] = fx_val(G[u]);
+      };
+      // H1 = sum over y of Gx P' + Gy D', H2 = of Gz P', by pairs of rows
+      long long H1[T2], H2[T2];
+#pragma unroll
+      for (int j = 0; j < T2; ++j) H1[j] = H2[j] = 0;
+      if (Q % 2) {
+        long long gx[K + 1], gy[K + 1], gz[K + 1];
+        row(Q / 2, gx, gy, gz);
+#pragma unroll
+        for (int u = 0, j = 0; u <= K; ++u) {
+          const Fx x = fx_split(gx[u]), yy = fx_split(gy[u]), z = fx_split(gz[u]);
+#pragma unroll
+          for (int v = 0; u + v <= K; ++v, ++j) {
+            FxAcc h1{0, 0}, h2{0, 0};
+            if (v % 2 == 0) {
+              fx_madt(h1, x, FT::W + v * Q + Q / 2);
+              fx_madt(h2, z, FT::W + v * Q + Q / 2);
+              H2[j] += fx_val(h2);
+            } else {
+              fx_madt(h1, yy, FT::D + v * Q + Q / 2);
+            }
+            H1[j] += fx_val(h1);
+          }
         }
       }
+#pragma unroll 1
+      for (int r = Q - Q / 2; r < Q; ++r) {
+        long long ax[K + 1], ay[K + 1], az[K + 1], bx[K + 1], by[K + 1], bz[K + 1];
+        row(r, ax, ay, az);
+        row(Q - 1 - r, bx, by, bz);
 #pragma unroll
-      for (int a = 0; a <= K; ++a) b2[CF::MT0 * C + (((ds * 5 + i) * KP + a) * Q + t2) * C + c] = m[a];
-    }
+        for (int u = 0, j = 0; u <= K; ++u) {
+          const Fx xs = fx_split(ax[u] + bx[u]), xd = fx_split(ax[u] - bx[u]);
+          const Fx ys_ = fx_split(ay[u] + by[u]), yd = fx_split(ay[u] - by[u]);
+          const Fx zs = fx_split(az[u] + bz[u]), zd = fx_split(az[u] - bz[u]);
+#pragma unroll
+          for (int v = 0; u + v <= K; ++v, ++j) {
+            FxAcc h1{0, 0}, h2{0, 0};
+            fx_madt(h1, v % 2 ? xd : xs, FT::W + v * Q + r);
+            if (v > 0) fx_madt(h1, v % 2 ? ys_ : yd, FT::D + v * Q + r);
+            fx_madt(h2, v % 2 ? zd : zs, FT::W + v * Q + r);
+            H1[j] += fx_val(h1);
+            H2[j] += fx_val(h2);
+          }
+        }
+      }
+      Fx wz[K + 1], dz[K + 1];
+#pragma unroll
+      for (int ww = 0; ww <= K; ++ww) {
+        wz[ww] = {c_fx[FT::W + ww * Q + qz][0], c_fx[FT::W + ww * Q + qz][1]};
+        dz[ww] = {c_fx[FT::D + ww * Q + qz][0], c_fx[FT::D + ww * Q + qz][1]};
+      }
+#pragma unroll
+      for (int u = 0, j = 0; u <= K; ++u)
+#pragma unroll
+        for (int v = 0; u + v <= K; ++v, ++j) {
+          const Fx h1 = fx_split(H1[j]), h2 = fx_split(H2[j]);
+#pragma unroll
+          for (int ww = 0; u + v + ww <= K; ++ww) {
+            FxAcc t{0, 0};
+            fx_mad(t, h1, wz[ww].h, wz[ww].l);
+            if (ww > 0) fx_mad(t, h2, dz[ww].h, dz[ww].l);
+            acc[mode_index(u, v, ww)] += fx_val(t);
+          }
+        }
   }
   __syncthreads();
-  // M[d*2+side][i][pair(a,b)] = +-(1/(4 dx_d)) sum_t2 Mt[a][t2] Pw(b, t2) -> b1
-  for (int it = tid; it < 30 * TP * C; it += kThreads) {
-    const int c = it % C, r = it / C, j = r % TP, i = (r / TP) % 5, ds = r / (5 * TP);
-    const int d = ds >> 1, side = ds & 1;
-    int a, b;
-    pair_uv<K>(j, a, b);
-    const T* mt = b2 + CF::MT0 * C + (((ds * 5 + i) * KP + a) * Q) * C + c;
-    T m = T(0);
+  // ------------------------- sum over the slices; R, or the FP64 stage update
+  long long* sAcc = reinterpret_cast<long long*>(smem_raw);
+  int* sExp = reinterpret_cast<int*>(sm64 + CF::EXPS);
+  float* sScr = reinterpret_cast<float*>(sm64 + CF::SCREEN);
 #pragma unroll
-    for (int t2 = 0; t2 < Q; ++t2) m += mt[t2 * C] * __ldg(P1W + b * Q + t2);
-    const T sc = (T)(0.25 * g.inv_dx[d]);
-    b1[it] = side == 0 ? m * sc : -(m * sc);
-  }
+  for (int l = 0; l < N; ++l) sAcc[((qz * 5 + i) * N + l) * C + c] = acc[l];
+  sExp[(qz * 5 + i) * C + c] = top >= kFxHuge ? 2 * kFxHuge : A;
   __syncthreads();
-  // dw/dt per (cell, variable, mode): volume + source + six faces
-  for (int it = tid; it < 5 * N * C; it += kThreads) {
-    const int c = it % C, r = it / C, l = r % N, i = r / N;
-    const long long cell = c0 + c;
-    int u, v, w;
-    mode_uvw(l, u, v, w);
-    const int j = pair_index(K, u, v);
-    const T* jr = b2 + ((i * TP + j) * Q) * C + c;
-    const T* ir2 = b2 + (((5 + i) * TP + j) * Q) * C + c;
-    T a = T(0);
+  int sh[Q], Am = 0;
 #pragma unroll
-    for (int qc = 0; qc < Q; ++qc) a += jr[qc * C] * __ldg(P1W + w * Q + qc) + ir2[qc * C] * __ldg(D1W + w * Q + qc);
-    if (FORCE && i > 0) {
-      const T* sr = b2 + (((10 + i - 1) * TP + j) * Q) * C + c;
+  for (int z = 0; z < Q; ++z) {
+    sh[z] = sExp[(z * 5 + i) * C + c];
+    Am = max(Am, sh[z]);
+  }
 #pragma unroll
-      for (int qc = 0; qc < Q; ++qc) a += sr[qc * C] * __ldg(P1W + w * Q + qc);
-    }
+  for (int z = 0; z < Q; ++z) sh[z] = min(Am - sh[z], 63);
+  float sab = 0.f;
+  if (live) {
+#pragma unroll 1
+    for (int l = qz; l < N; l += Q) {
+      const size_t at = (size_t)(i * N + l) * nc + cell;
+      long long s = 0;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int e = d == 0 ? u : (d == 1 ? v : w);
-      const int pa = d == 0 ? v : u, pb = d == 2 ? v : w;
-      const int jf = pair_index(K, pa, pb);
-#pragma unroll
-      for (int side = 0; side < 2; ++side)
-        a += b1[(((d * 2 + side) * 5 + i) * TP + jf) * C + c] * __ldg(tab + TB::FEND + side * KP + e);
-    }
-    if (cell < nc) {
-      const size_t at = (size_t)r * nc + cell;
+      for (int z = 0; z < Q; ++z) s += sAcc[((z * 5 + i) * N + l) * C + c] >> sh[z];
+      const double a = Am < kFxHuge ? fx_to_double(s, Am + p4) : __longlong_as_double(0x7ff8000000000000LL);
       if (MODE == MODE_RHS) {
-        R[at] = -(double)a;
+        R[at] = -a;
       } else {
-        const double vv = st.a0 * st.y0[at] + st.b0 * (st.ys[at] + st.dt * (double)a);
-        st.out[at] = vv;
-        if constexpr (sizeof(T) == 4) st.yf[at] = (float)vv;
-        sV[r * C + c] = vv;
+        // the first stage (a0 = 0, b0 = 1) does not read y_0
+        double v = fma(st.dt, a, __ldcg(st.ys + at));
+        if (st.a0 != 0.0) v = st.a0 * __ldcg(st.y0 + at) + st.b0 * v;
+        st.out[at] = v;
+        if (l == 0) sScr[(Q * 5 + i) * C + c] = f64_to_f32_q(v);
+        else sab = fmaf(abs_up(v), c_tab32[(g.lim_vol ? TB::LMAXV : TB::LMAX) + l], sab);
       }
     }
   }
   if (MODE == MODE_RHS) return;
+  // limiter screen of the next stage's input (FP32, sufficient); cells that
+  // fail it are queued for the full limiter
+  sScr[(qz * 5 + i) * C + c] = sab * (1.f + 1e-5f);
   __syncthreads();
-  // limiter screen of the next stage's input (FP64); cells that fail it are
-  // queued for the full limiter
-  for (int it = tid; it < 5 * C; it += kThreads) {
-    const int c = it % C, i = it / C;
-    if (c0 + c >= nc) continue;
-    const double* row = sV + (i * N) * C + c;
-    double sa = 0.0;
-    bool fin = isfinite(row[0]);
-    for (int l = 1; l < N; ++l) {
-      sa += fabs(row[l * C]) * __ldg(tab64 + (g.lim_vol ? TB::LMAXV : TB::LMAX) + l);
-      fin &= isfinite(row[l * C]);
-    }
-    sM[it] = fin ? row[0] : __longlong_as_double(0x7ff8000000000000LL);
-    sA[it] = sa;
-  }
-  __syncthreads();
-  if (tid < C && c0 + tid < nc) {
-    double m[5], a[5];
-    bool fin = true;
+  if (tid < C && live) {
+    float m[5], s[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      m[i] = sM[i * C + tid];
-      a[i] = sA[i * C + tid];
-      fin &= isfinite(m[i]);
+    for (int v = 0; v < 5; ++v) {
+      m[v] = sScr[(Q * 5 + v) * C + tid];
+      s[v] = 0.f;
+#pragma unroll
+      for (int z = 0; z < Q; ++z) s[v] += sScr[(z * 5 + v) * C + tid];
     }
-    if (!limiter_screen<K>(m, a, fin, g.gamma, g.eps_rho, g.eps_p)) {
+    if (!screen_f32(m, s, (float)gm1, (float)g.eps_rho, (float)g.eps_p)) {
       const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
-      st.list[slot] = (int)(c0 + tid);
+      st.list[slot] = (int)cell;
     }
   }
 }
