@@ -31,54 +31,170 @@ __device__ __forceinline__ double scaled_legendre(int u, double x) {
   return sqrt(2.0 * u + 1.0) * p;
 }
 
-// out[(Z * M + Y) * M + X] = m_comp / rho of the state polynomial at the
-// centre of sub-cell (X % sub, Y % sub, Z % sub) of cell (X, Y, Z) / sub
-__global__ void sample_kernel(const double* __restrict__ y, int k, int n, int sub, int comp, double* __restrict__ out) {
-  const int N = nmodes(k), M = n * sub;
-  const long long total = (long long)M * M * M, nc = (long long)n * n * n;
+// Samples of the state polynomial at the centres of sub^3 sub-cells per cell,
+// sum-factorised in 64-bit fixed point (dg_common.cuh): a thread takes one cell
+// and one z of its sub-cells (lanes: cells along x, so that a row of samples is
+// written in one piece), contracts the coefficients along z once, along y per
+// sub-cell row and along x per sample. tab: Pt_u at the sub-cell centres in
+// units of 2^-58, [u][8]. What bounds it is the integer pipe and, for the
+// velocity, the 4 FP64 operations of a division per sample; with the Legendre
+// recurrences and the dense sum in FP64 per sample, 256^3 samples of one
+// component took 5.72 ms, now 0.215.
+constexpr int kMaxSub = 8;
+
+__device__ __forceinline__ void sub_table(int k, int sub, int (*tab)[2]) {
+  for (int j = threadIdx.x; j < (k + 1) * kMaxSub; j += blockDim.x) {
+    const int u = j / kMaxSub, s = j % kMaxSub;
+    const Fx c = fx_split(s < sub ? fx_from(scaled_legendre(u, -1.0 + (2.0 * s + 1.0) / sub), 1025) : 0);
+    tab[j][0] = c.h;
+    tab[j][1] = c.l;
+  }
+  __syncthreads();
+}
+
+template <int K>
+struct SubCell {
+  static constexpr int N = nmodes(K), T = (K + 1) * (K + 2) / 2;
+  Fx a1[T], a2[K + 1];
+  int B;
+  // the variable's coefficients (rows nc apart) contracted along z
+  __device__ __forceinline__ void load(const double* __restrict__ y, size_t nc, const int (*tab)[2], int sz) {
+    double w[N];
+#pragma unroll
+    for (int l = 0; l < N; ++l) w[l] = __ldg(y + (size_t)l * nc);
+    B = fx_bound<K>(w);
+#pragma unroll
+    for (int u = 0, j = 0; u <= K; ++u)
+#pragma unroll
+      for (int v = 0; u + v <= K; ++v, ++j) {
+        FxAcc s{0, 0};
+#pragma unroll
+        for (int ww = 1; u + v + ww <= K; ++ww)
+          fx_mad(s, fx_split(fx_from(w[mode_index(u, v, ww)], B)), tab[ww * kMaxSub + sz][0], tab[ww * kMaxSub + sz][1]);
+        a1[j] = fx_split(fx_val(s) + fx_from(w[mode_index(u, v, 0)], B));
+      }
+  }
+  __device__ __forceinline__ void row(const int (*tab)[2], int sy) {
+#pragma unroll
+    for (int u = 0, j = 0; u <= K; ++u) {
+      FxAcc s{0, 0};
+      const long long x0 = fx_join(a1[j]);
+      ++j;
+#pragma unroll
+      for (int v = 1; u + v <= K; ++v, ++j) fx_mad(s, a1[j], tab[v * kMaxSub + sy][0], tab[v * kMaxSub + sy][1]);
+      a2[u] = fx_split(fx_val(s) + x0);
+    }
+  }
+  __device__ __forceinline__ long long at(const int (*tab)[2], int sx) const {
+    FxAcc s{0, 0};
+#pragma unroll
+    for (int u = 1; u <= K; ++u) fx_mad(s, a2[u], tab[u * kMaxSub + sx][0], tab[u * kMaxSub + sx][1]);
+    return fx_val(s) + fx_join(a2[0]);
+  }
+  __device__ __forceinline__ double value(const int (*tab)[2], int sx) const {
+    return B < kFxHuge ? fx_to_double(at(tab, sx), B) : __longlong_as_double(0x7ff8000000000000LL);
+  }
+};
+
+// item e = ((iz n + iy) sub + sz) n + ix
+__device__ __forceinline__ void sub_item(long long e, int n, int sub, int& ix, int& iy, int& iz, int& sz) {
+  ix = (int)(e % n);
+  const long long r = e / n;
+  sz = (int)(r % sub);
+  const int yz = (int)(r / sub);
+  iy = yz % n;
+  iz = yz / n;
+}
+
+template <int K>
+__device__ __forceinline__ void sample_cells(const double* __restrict__ y, int n, int sub, int comp,
+                                             double* __restrict__ out, const int (*tab)[2]) {
+  const int M = n * sub;
+  const long long total = (long long)n * n * n * sub, nc = (long long)n * n * n;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
-    const int X = (int)(e % M), Y = (int)((e / M) % M), Z = (int)(e / ((long long)M * M));
-    const long long cell = ((long long)(Z / sub) * n + Y / sub) * n + X / sub;
-    const double xi[3] = {-1.0 + (2.0 * (X % sub) + 1.0) / sub, -1.0 + (2.0 * (Y % sub) + 1.0) / sub,
-                          -1.0 + (2.0 * (Z % sub) + 1.0) / sub};
-    double P[3][4];
-    for (int a = 0; a < 3; ++a)
-      for (int u = 0; u <= k; ++u) P[a][u] = scaled_legendre(u, xi[a]);
-    double rho = 0.0, m = 0.0;
-    for (int l = 0; l < N; ++l) {
-      int u, v, w;
-      mode_uvw(l, u, v, w);
-      const double phi = P[0][u] * P[1][v] * P[2][w];
-      rho += y[(size_t)l * nc + cell] * phi;
-      m += y[(size_t)((1 + comp) * N + l) * nc + cell] * phi;
+    int ix, iy, iz, sz;
+    sub_item(e, n, sub, ix, iy, iz, sz);
+    const long long cell = ((long long)iz * n + iy) * n + ix;
+    SubCell<K> r, m;
+    r.load(y + cell, nc, tab, sz);
+    m.load(y + (size_t)((1 + comp) * SubCell<K>::N) * nc + cell, nc, tab, sz);
+    double* o = out + ((size_t)(iz * sub + sz) * M + (size_t)iy * sub) * M + (size_t)ix * sub;
+#pragma unroll 1
+    for (int sy = 0; sy < sub; ++sy, o += M) {
+      r.row(tab, sy);
+      m.row(tab, sy);
+#pragma unroll 2
+      for (int sx = 0; sx < sub; ++sx) o[sx] = m.value(tab, sx) * rcp64(r.value(tab, sx));
     }
-    out[e] = m / rho;
   }
 }
 
+// out[(Z * M + Y) * M + X] = m_comp / rho of the state polynomial at the
+// centre of sub-cell (X % sub, Y % sub, Z % sub) of cell (X, Y, Z) / sub
+__global__ void __launch_bounds__(256) sample_kernel(const double* __restrict__ y, int k, int n, int sub, int comp,
+                                                     double* __restrict__ out) {
+  __shared__ int tab[4 * kMaxSub][2];
+  sub_table(k, sub, tab);
+  if (k == 0) sample_cells<0>(y, n, sub, comp, out, tab);
+  else if (k == 1) sample_cells<1>(y, n, sub, comp, out, tab);
+  else if (k == 2) sample_cells<2>(y, n, sub, comp, out, tab);
+  else sample_cells<3>(y, n, sub, comp, out, tab);
+}
+
+// shell round(sqrt(k2)) of an integer k2: the b with b^2 - b < k2 <= b^2 + b
+__device__ __forceinline__ int shell_of(long long k2) {
+  long long b = (long long)sqrtf((float)k2);
+  while (b > 0 && b * b - b >= k2) --b;
+  while (b * b + b < k2) ++b;
+  return (int)b;
+}
+
 // shell sums of the half spectrum [M][M][M/2 + 1]: each element stands for
-// itself and (unless its last index is 0 or M/2) its conjugate partner
-__global__ void bin_kernel(const double2* __restrict__ sp, int M, int nb, double* __restrict__ bins) {
+// itself and (unless its last index is 0 or M/2) its conjugate partner. A
+// thread takes kRun consecutive elements of a row (one 128-byte line), along
+// which the shell never falls, and adds one sum per shell to its warp's copy of
+// the bins where there is room for one per warp (copies; shared memory holds nb
+// doubles per copy): a double has no native shared-memory atomic, and with one
+// addition per element on one copy 256^3 took 0.431 ms per component, now 0.137.
+constexpr int kRun = 8;
+__global__ void __launch_bounds__(256) bin_kernel(const double2* __restrict__ sp, int M, int nb,
+                                                  double* __restrict__ bins, int copies = 1) {
   extern __shared__ double sh[];
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) sh[b] = 0.0;
+  for (int b = threadIdx.x; b < nb * copies; b += blockDim.x) sh[b] = 0.0;
   __syncthreads();
-  const int H = M / 2 + 1;
-  const long long total = (long long)M * M * H;
+  double* mine = sh + (size_t)((int)(threadIdx.x >> 5) % copies) * nb;
+  const int H = M / 2 + 1, chunks = (H + kRun - 1) / kRun;
+  const long long total = (long long)M * M * chunks;
   const double norm = 1.0 / ((double)M * M * M) / ((double)M * M * M);
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(e % H), b = (int)((e / H) % M), a = (int)(e / ((long long)H * M));
-    const int kx = c, ky = b <= M / 2 ? b : b - M, kz = a <= M / 2 ? a : a - M;
-    const double kk = sqrt((double)kx * kx + (double)ky * ky + (double)kz * kz);
-    const int bin = (int)floor(kk + 0.5);
-    const double w = (c == 0 || (M % 2 == 0 && c == M / 2)) ? 1.0 : 2.0;
-    const double2 z = sp[e];
-    if (bin < nb) atomicAdd(&sh[bin], w * (z.x * z.x + z.y * z.y) * norm);
+    const int first = (int)(e % chunks) * kRun, last = min(first + kRun, H);
+    const long long row = e / chunks;
+    const int b = (int)(row % M), a = (int)(row / M);
+    const int ky = b <= M / 2 ? b : b - M, kz = a <= M / 2 ? a : a - M;
+    const long long yz = (long long)ky * ky + (long long)kz * kz;
+    const double2* z = sp + row * H;
+    int run = -1;
+    double p = 0.0;
+    for (int c = first; c < last; ++c) {
+      const int bin = shell_of(yz + (long long)c * c);
+      if (bin != run) {
+        if (run >= 0 && run < nb) atomicAdd(&mine[run], p);
+        run = bin;
+        p = 0.0;
+      }
+      const double w = (c == 0 || (M % 2 == 0 && c == M / 2)) ? norm : 2.0 * norm;
+      p = fma(w, fma(z[c].x, z[c].x, z[c].y * z[c].y), p);
+    }
+    if (run >= 0 && run < nb) atomicAdd(&mine[run], p);
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < nb; b += blockDim.x)
-    if (sh[b] != 0.0) atomicAdd(&bins[b], sh[b]);
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+    double s = 0.0;
+    for (int j = 0; j < copies; ++j) s += sh[(size_t)j * nb + b];
+    if (s != 0.0) atomicAdd(&bins[b], s);
+  }
 }
 
 // cuFFT plan of an M^3 D2Z transform with a caller-owned work area
@@ -91,44 +207,80 @@ cufftResult make_plan(int M, cufftHandle* plan, size_t* ws) {
   return r;
 }
 
-// histogram of ln(rho) of the state polynomial at the sub-cell centres:
+// Histogram of ln(rho) of the state polynomial at the sub-cell centres:
 // counts[0] below lo (and non-positive or non-finite densities),
 // counts[1 + j] for floor((ln rho - lo) / (hi - lo) * nb) = j, counts[nb + 1]
-// at or above hi; integer counts (order-independent)
-__global__ void density_hist_kernel(const double* __restrict__ y, int k, int n, int sub, double lo, double hi, int nb,
-                                    unsigned long long* __restrict__ counts) {
-  extern __shared__ unsigned int shc[];
-  for (int b = threadIdx.x; b < nb + 2; b += blockDim.x) shc[b] = 0u;
-  __syncthreads();
-  const int N = nmodes(k), M = n * sub;
-  const long long total = (long long)M * M * M, nc = (long long)n * n * n;
+// at or above hi; integer counts (order-independent). The bin comes from an
+// FP32 logarithm; where its error could reach a bin's edge, from FP64 as the
+// definition has it. A thread's samples mostly fall into one bin after the
+// other: runs are counted before they go to the shared histogram. The FP64
+// logarithm and the dense sum of every sample took 6.54 ms for 256^3 samples,
+// now 0.133.
+__device__ __forceinline__ int density_bin(long long r, int B, double lo, double hi, int nb, float flo, float scale,
+                                           float slack) {
+  if (B >= kFxHuge || r <= 0) return 0;
+  // ln r from the significand in [1, 2) and the exponent
+  const int lz = clz64((unsigned long long)r);
+  const unsigned m = (unsigned)(((unsigned long long)r << lz) >> 32);
+  const int ex = B - 1083 + 63 - lz;
+  const float f = __uint_as_float(0x3f800000u | ((m >> 8) & 0x7fffffu));
+  const float s = fmaf((float)ex, 0.69314718056f, logf(f));
+  const float t = (s - flo) * scale, e = slack + fabsf(s) * scale * 1e-6f, j = floorf(t);
+  if (t - j > e && j + 1.f - t > e && t > -1e6f && t < 1e6f) return t < 0.f ? 0 : (t >= (float)nb ? nb + 1 : 1 + (int)j);
+  const double rho = fx_to_double(r, B);
+  if (!(rho > 0.0)) return 0;
+  const double sv = log(rho);
+  if (sv >= hi) return nb + 1;
+  if (!(sv >= lo)) return 0;
+  const int k = (int)floor((sv - lo) / (hi - lo) * nb);
+  return 1 + (k < nb ? k : nb - 1);
+}
+
+template <int K>
+__device__ __forceinline__ void hist_cells(const double* __restrict__ y, int n, int sub, double lo, double hi, int nb,
+                                           const int (*tab)[2], unsigned int* shc) {
+  const long long total = (long long)n * n * n * sub, nc = (long long)n * n * n;
+  // FP32 bin position (s - lo) scale; the rounding of s, lo and scale stays
+  // below 1e-6 (|s| + |lo|) scale, to which `slack` adds that of the products
+  const float flo = (float)lo, scale = (float)(nb / (hi - lo));
+  const float slack = (fabsf(flo) + 1.f) * scale * 1e-6f + (float)nb * 1e-6f + 1e-6f;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
-    const int X = (int)(e % M), Y = (int)((e / M) % M), Z = (int)(e / ((long long)M * M));
-    const long long cell = ((long long)(Z / sub) * n + Y / sub) * n + X / sub;
-    const double xi[3] = {-1.0 + (2.0 * (X % sub) + 1.0) / sub, -1.0 + (2.0 * (Y % sub) + 1.0) / sub,
-                          -1.0 + (2.0 * (Z % sub) + 1.0) / sub};
-    double P[3][4];
-    for (int a = 0; a < 3; ++a)
-      for (int u = 0; u <= k; ++u) P[a][u] = scaled_legendre(u, xi[a]);
-    double rho = 0.0;
-    for (int l = 0; l < N; ++l) {
-      int u, v, w;
-      mode_uvw(l, u, v, w);
-      rho += y[(size_t)l * nc + cell] * (P[0][u] * P[1][v] * P[2][w]);
-    }
-    int b = 0;
-    if (rho > 0.0 && isfinite(rho)) {
-      const double sv = log(rho);
-      if (sv >= hi) {
-        b = nb + 1;
-      } else if (sv >= lo) {
-        const int j = (int)floor((sv - lo) / (hi - lo) * nb);
-        b = 1 + (j < nb ? j : nb - 1);
+    int ix, iy, iz, sz;
+    sub_item(e, n, sub, ix, iy, iz, sz);
+    SubCell<K> r;
+    r.load(y + ((long long)iz * n + iy) * n + ix, nc, tab, sz);
+    int run = -1;
+    unsigned count = 0;
+#pragma unroll 1
+    for (int sy = 0; sy < sub; ++sy) {
+      r.row(tab, sy);
+#pragma unroll 2
+      for (int sx = 0; sx < sub; ++sx) {
+        const int b = density_bin(r.at(tab, sx), r.B, lo, hi, nb, flo, scale, slack);
+        if (b != run) {
+          if (count) atomicAdd(&shc[run], count);
+          run = b;
+          count = 0;
+        }
+        ++count;
       }
     }
-    atomicAdd(&shc[b], 1u);
+    atomicAdd(&shc[run], count);
   }
+}
+
+__global__ void __launch_bounds__(256) density_hist_kernel(const double* __restrict__ y, int k, int n, int sub,
+                                                           double lo, double hi, int nb,
+                                                           unsigned long long* __restrict__ counts) {
+  extern __shared__ unsigned int shc[];
+  __shared__ int tab[4 * kMaxSub][2];
+  for (int b = threadIdx.x; b < nb + 2; b += blockDim.x) shc[b] = 0u;
+  sub_table(k, sub, tab);
+  if (k == 0) hist_cells<0>(y, n, sub, lo, hi, nb, tab, shc);
+  else if (k == 1) hist_cells<1>(y, n, sub, lo, hi, nb, tab, shc);
+  else if (k == 2) hist_cells<2>(y, n, sub, lo, hi, nb, tab, shc);
+  else hist_cells<3>(y, n, sub, lo, hi, nb, tab, shc);
   __syncthreads();
   for (int b = threadIdx.x; b < nb + 2; b += blockDim.x)
     if (shc[b]) atomicAdd(&counts[b], (unsigned long long)shc[b]);
@@ -140,7 +292,9 @@ cudaError_t density_pdf(int k, const double* y, int n, int sub, double lo, doubl
                         unsigned long long* counts_dev, long long* counts_host, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(counts_dev, 0, sizeof(unsigned long long) * (nb + 2), s);
   if (e != cudaSuccess) return e;
-  density_hist_kernel<<<1024, 256, sizeof(unsigned int) * (nb + 2), s>>>(y, k, n, sub, lo, hi, nb, counts_dev);
+  const long long items = (long long)n * n * n * sub;
+  const unsigned grid = (unsigned)((items + 255) / 256 < 152 * 16 ? (items + 255) / 256 : 152 * 16);
+  density_hist_kernel<<<grid, 256, sizeof(unsigned int) * (nb + 2), s>>>(y, k, n, sub, lo, hi, nb, counts_dev);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   e = cudaMemcpyAsync(counts_host, counts_dev, sizeof(unsigned long long) * (nb + 2), cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return e;
@@ -202,11 +356,15 @@ cudaError_t velocity_spectrum(int k, const double* y, int n, int sub, void* work
   cudaError_t e = cudaSuccess;
   if ((r = cufftSetWorkArea(plan, area)) == CUFFT_SUCCESS) r = cufftSetStream(plan, s);
   if (r == CUFFT_SUCCESS) e = cudaMemsetAsync(bins, 0, sizeof(double) * nb, s);
+  // a copy of the bins per warp while the eight fit 48 KB
+  const int copies = (size_t)nb * sizeof(double) * 8 <= 48 * 1024 ? 8 : 1;
+  const long long items = (long long)n * n * n * sub;
+  const unsigned grid = (unsigned)((items + 255) / 256 < 152 * 16 ? (items + 255) / 256 : 152 * 16);
   for (int comp = 0; comp < 3 && r == CUFFT_SUCCESS && e == cudaSuccess; ++comp) {
-    sample_kernel<<<2048, 256, 0, s>>>(y, k, n, sub, comp, real);
+    sample_kernel<<<grid, 256, 0, s>>>(y, k, n, sub, comp, real);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
     if ((r = cufftExecD2Z(plan, real, reinterpret_cast<cufftDoubleComplex*>(cplx))) != CUFFT_SUCCESS) break;
-    bin_kernel<<<1024, 256, sizeof(double) * nb, s>>>(cplx, M, nb, bins);
+    bin_kernel<<<152 * 4, 256, sizeof(double) * nb * copies, s>>>(cplx, M, nb, bins, copies);
     e = cudaGetLastError();
   }
   if (r == CUFFT_SUCCESS && e == cudaSuccess)
