@@ -338,7 +338,7 @@ int dg_indicator_adam(float* params, float* m, float* v, const float* grads, int
  * The numerical flux is always HLLC (there is no context, so dg_set_flux
  * does not apply). FP64: the kernels of dg_rhs, same results. DG_PREC_MIXED:
  * the separate FP32 face and volume kernels, within FP32 rounding of
- * dg_rhs (which runs the fused stage kernel at degree 2).
+ * dg_rhs (which runs the fused stage kernel at degrees 1 to 3).
  * Device-side errors are not reported: a non-finite y gives a non-finite R
  * and DG_OK, so check R where that matters; the return value covers the
  * arguments, the size limit and CUDA launch errors only. */

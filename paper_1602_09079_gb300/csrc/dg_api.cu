@@ -198,8 +198,10 @@ Launchers launchers_for(int k) {
   }
 }
 
-// fused FP32-mixed stage kernels exist for degrees 2 and 3
+// fused FP32-mixed stage kernels: degrees 1 to 3 (at degree 0 a cell has no
+// integral to fuse)
 FusedLaunchers fused_for(int k) {
+  if (k == 1) return fused_launchers_k1();
   if (k == 2) return fused_launchers_k2();
   if (k == 3) return fused_launchers_k3();
   FusedLaunchers L{};
@@ -342,7 +344,8 @@ struct dg_ctx {
   Ctrl* ctrl = nullptr;
   double* part = nullptr;
   double* modes_dev = nullptr;
-  double* sums = nullptr;  // 8 doubles
+  int cfl_slot = 0;            // which of the control block's CFL maxima the next reduction uses
+  bool queue_open = false;     // n_flag may not be 0 (see open_queue)
   double* ybuf = nullptr;
   int* list = nullptr;
   int* list2 = nullptr;
@@ -378,7 +381,7 @@ struct dg_ctx {
 namespace {
 
 struct Layout {
-  size_t ctrl, part, modes, sums, ybuf, list, list2, yf, fh, field, base_end, full_end;
+  size_t ctrl, part, modes, ybuf, list, list2, yf, fh, field, base_end, full_end;
 };
 
 Layout layout_of(const dg_ctx* c) {
@@ -392,8 +395,6 @@ Layout layout_of(const dg_ctx* c) {
   o += align256(sizeof(double) * npart);
   L.modes = o;
   o += align256(sizeof(double) * 9 * kMaxForce);
-  L.sums = o;
-  o += align256(sizeof(double) * 8);
   L.ybuf = o;
   o += align256(sizeof(double) * 5 * c->N * nc);
   L.list = o;
@@ -443,6 +444,14 @@ int sync_and_check(dg_ctx* c, Ctrl* host_copy) {
     DG_CUDA(cudaStreamSynchronize(c->stream));
   }
   return err_to_status(h.err);
+}
+
+// Cells are about to be queued: the queue is empty unless an earlier call
+// failed between the kernel that queued cells and the limiter that empties it.
+int open_queue(dg_ctx* c) {
+  if (c->queue_open) DG_CUDA(cudaMemsetAsync(&c->ctrl->n_flag, 0, sizeof(unsigned), c->stream));
+  c->queue_open = true;
+  return DG_OK;
 }
 
 int set_device(const dg_ctx* c) { return cuda_ok(cudaSetDevice(c->device)); }
@@ -550,7 +559,7 @@ int fused_step(dg_ctx* c, double dt, bool force) {
     a.b0_d = b0[s];
     a.y0 = c->y;
     a.stage = s + 1;
-    DG_CUDA(cudaMemsetAsync(&c->ctrl->n_flag, 0, sizeof(unsigned), c->stream));
+    DG_TRY(open_queue(c));
     DG_TRY(launch(c, KC_VOLUME, [&] { return c->fz.run(force, c->flux, c->geo, a, c->stream); }));
     float* yf = s == 2 ? c->yf : nullptr;
     const double* y0 = s < 2 ? c->y : nullptr;
@@ -571,6 +580,7 @@ int fused_step(dg_ctx* c, double dt, bool force) {
                                 c->stream);
       }, 2));
     }
+    c->queue_open = false;
     ys = out;
   }
   c->limited = true;
@@ -671,7 +681,8 @@ int dg_bind(dg_ctx* c, double* y_dev, void* scratch_dev, size_t scratch_bytes, v
   c->ctrl = reinterpret_cast<Ctrl*>(c->scratch + L.ctrl);
   c->part = reinterpret_cast<double*>(c->scratch + L.part);
   c->modes_dev = reinterpret_cast<double*>(c->scratch + L.modes);
-  c->sums = reinterpret_cast<double*>(c->scratch + L.sums);
+  c->cfl_slot = 0;
+  c->queue_open = false;
   c->ybuf = reinterpret_cast<double*>(c->scratch + L.ybuf);
   c->list = reinterpret_cast<int*>(c->scratch + L.list);
   c->list2 = reinterpret_cast<int*>(c->scratch + L.list2);
@@ -828,7 +839,7 @@ int dg_step(dg_ctx* c, double dt) {
   for (int s = 0; s < 3; ++s) {
     double* out = s < 2 ? c->ybuf : c->y;
     DG_TRY(launch(c, KC_FACE, [&] { return c->fn.face(c->prec, c->flux, ys, yf, c->fh, c->geo, c->ctrl, c->stream); }));
-    DG_CUDA(cudaMemsetAsync(&c->ctrl->n_flag, 0, sizeof(unsigned), c->stream));
+    DG_TRY(open_queue(c));
     DG_TRY(launch(c, KC_VOLUME, [&] {
       return c->fn.volume_stage(c->prec, force, c->fh, c->field, c->geo, ys, c->y, out, a0[s], b0[s], dt, c->list,
                                 yf, c->ctrl, c->stream);
@@ -851,6 +862,7 @@ int dg_step(dg_ctx* c, double dt) {
                                 c->stream);
       }, 2));
     }
+    c->queue_open = false;
     ys = out;
   }
   c->limited = true;
@@ -878,13 +890,14 @@ int dg_cfl_dt(dg_ctx* c, double courant, double* dt_out) {
   DG_TRY(need_bound(c));
   if (!dt_out || !(courant > 0.0)) return DG_ERR_ARG;
   DG_TRY(set_device(c));
-  DG_CUDA(cudaMemsetAsync(&c->ctrl->cfl_max_bits, 0, sizeof(unsigned long long), c->stream));
-  DG_TRY(launch(c, KC_CFL, [&] { return c->fn.cfl(c->y, c->geo, c->ctrl, c->stream); }));
+  const int slot = c->cfl_slot;
+  c->cfl_slot ^= 1;
+  DG_TRY(launch(c, KC_CFL, [&] { return c->fn.cfl(c->y, c->geo, c->ctrl, slot, c->stream); }));
   Ctrl h{};
   int st = sync_and_check(c, &h);
   if (st != DG_OK) return st;
   double smax;
-  std::memcpy(&smax, &h.cfl_max_bits, sizeof(double));
+  std::memcpy(&smax, slot ? &h.cfl_max_bits2 : &h.cfl_max_bits, sizeof(double));
   if (!(smax > 0.0)) return DG_ERR_POSITIVITY;
   // C min(1/(2k+1), w1/2) with w1 = 1 (m = 2 GLL points), 1/3 (m = 3)
   const double w1 = gll_m(c->k) == 2 ? 1.0 : 1.0 / 3.0;
@@ -959,7 +972,7 @@ int dg_energy_reset(dg_ctx* c, double c_iso, double rho0, double* dissipated) {
   // keep the FP32 shadow current if it is (energy rows and limited cells)
   float* yf = (uses_shadow(c) && c->shadow_valid) ? c->yf : nullptr;
   if (!yf) c->shadow_valid = false;
-  DG_CUDA(cudaMemsetAsync(&c->ctrl->n_flag, 0, sizeof(unsigned), c->stream));
+  DG_TRY(open_queue(c));
   DG_TRY(launch(c, KC_RESET, [&] {
     return c->fn.energy_reset(c->prec, c->y, c->geo, c2g, 1.0 / rho0, c->part, &n_part, c->list, c->ctrl, yf,
                               c->stream);
@@ -970,17 +983,17 @@ int dg_energy_reset(dg_ctx* c, double c_iso, double rho0, double* dissipated) {
     return c->fn.limit_list(c->y, c->list, &c->ctrl->n_flag, c->geo, c->ctrl, 0, yf, nullptr, nullptr, c->list2,
                                 c->stream);
   }, 2));
+  c->queue_open = false;
   c->limited = true;
   if (dissipated) {
     const double vol = c->geo.dx[0] * c->geo.dx[1] * c->geo.dx[2];
     DG_TRY(launch(c, KC_OTHER, [&] {
-      sum_rows_kernel<<<1, 256, 0, c->stream>>>(c->part, n_part, vol, c->sums);
+      sum_rows_kernel<<<1, 256, 0, c->stream>>>(c->part, n_part, vol, c->ctrl->sums);
       return cudaGetLastError();
     }));
-    double h = 0.0;
-    DG_CUDA(cudaMemcpyAsync(&h, c->sums, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    int st = sync_and_check(c, nullptr);
-    *dissipated = h;
+    Ctrl h{};
+    int st = sync_and_check(c, &h);
+    *dissipated = h.sums[0];
     return st;
   }
   return DG_OK;
@@ -990,24 +1003,25 @@ int dg_diagnostics(dg_ctx* c, double* out3) {
   DG_TRY(need_bound(c));
   if (!out3) return DG_ERR_ARG;
   DG_TRY(set_device(c));
-  long long nb = (c->geo.nc + 255) / 256;
-  const int G = (int)(nb < kRedBlocks ? nb : kRedBlocks);
   const int force = c->n_force > 0 ? 1 : 0;
+  // a thread per cell, or per cell and direction of the driving; three partial
+  // sums of each block fit the area of kRedBlocks blocks' ten
+  long long nb = ((force ? 3 : 1) * c->geo.nc + 255) / 256;
+  const int G = (int)(nb < 3 * kRedBlocks ? nb : 3 * kRedBlocks);
   DG_TRY(launch(c, KC_OTHER, [&] {
     return c->fn.diagnostics(c->prec, c->y, c->field, force, c->geo, c->part, G, c->stream);
   }));
   const double vol = c->geo.dx[0] * c->geo.dx[1] * c->geo.dx[2];
   DG_TRY(launch(c, KC_OTHER, [&] {
-    sum_rows_kernel<<<3, 256, 0, c->stream>>>(c->part, G, vol, c->sums);
+    sum_rows_kernel<<<3, 256, 0, c->stream>>>(c->part, G, vol, c->ctrl->sums);
     return cudaGetLastError();
   }));
-  double h[3];
-  DG_CUDA(cudaMemcpyAsync(h, c->sums, sizeof(double) * 3, cudaMemcpyDeviceToHost, c->stream));
-  const int st = sync_and_check(c, nullptr);
+  Ctrl h{};
+  const int st = sync_and_check(c, &h);
   if (st != DG_OK) return st;
-  out3[0] = std::sqrt(h[0] / (c->L[0] * c->L[1] * c->L[2]));
-  out3[1] = h[1];
-  out3[2] = h[2];
+  out3[0] = std::sqrt(h.sums[0] / (c->L[0] * c->L[1] * c->L[2]));
+  out3[1] = h.sums[1];
+  out3[2] = h.sums[2];
   return DG_OK;
 }
 
@@ -1074,11 +1088,13 @@ int dg_totals(dg_ctx* c, double* out5) {
   }));
   const double vol = c->geo.dx[0] * c->geo.dx[1] * c->geo.dx[2];
   DG_TRY(launch(c, KC_OTHER, [&] {
-    sum_rows_kernel<<<5, 256, 0, c->stream>>>(c->part, G, vol, c->sums);
+    sum_rows_kernel<<<5, 256, 0, c->stream>>>(c->part, G, vol, c->ctrl->sums);
     return cudaGetLastError();
   }));
-  DG_CUDA(cudaMemcpyAsync(out5, c->sums, sizeof(double) * 5, cudaMemcpyDeviceToHost, c->stream));
-  return sync_and_check(c, nullptr);
+  Ctrl h{};
+  const int st = sync_and_check(c, &h);
+  std::memcpy(out5, h.sums, sizeof(double) * 5);
+  return st;
 }
 
 int dg_check(dg_ctx* c) {

@@ -94,7 +94,9 @@ enum : unsigned {
   ERRB_NEWTON = 4u,
 };
 
-// Control block at the start of the scratch buffer.
+// Control block at the start of the scratch buffer. The queue counters are zero
+// between the calls that use them: every stage (and the energy reset) clears
+// n_deep before its cells are queued, the limiter's last pass clears n_flag.
 struct Ctrl {
   unsigned long long cfl_max_bits;  // max over cells of the wave-speed sum (bits of a double >= 0)
   unsigned int err;                 // sticky ERRB_* bits
@@ -104,7 +106,8 @@ struct Ctrl {
   unsigned int n_deep;              // queued cells the FP32 point screen does not clear
   unsigned long long n_queued_total;  // cells that failed the limiter screen (all stages)
   unsigned long long n_full_total;    // cells that went through the full limiter
-  double pad1[2];
+  unsigned long long cfl_max_bits2;   // the maximum of every second CFL reduction; each clears the other's
+  double sums[8];                     // results of the host-facing sums, read back with the error word
 };
 
 struct Geo {
@@ -407,6 +410,15 @@ __device__ __forceinline__ long long fx_from(double x, int B) {
   unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 40) | ((unsigned long long)lo << 8);
   m >>= d;
   return (hi >> 31) ? -(long long)m : (long long)m;
+}
+
+// the same of a binary32 value (biased exponent + 896 <= B)
+__device__ __forceinline__ long long fx_from(float x, int B) {
+  const unsigned u = __float_as_uint(x);
+  const int e = (int)((u >> 23) & 0xffu);
+  const int d = e ? min(B - 896 - e, 63) : 63;
+  const unsigned long long m = ((unsigned long long)((u & 0x7fffffu) | 0x800000u) << 37) >> d;
+  return (u >> 31) ? -(long long)m : (long long)m;
 }
 
 __device__ __forceinline__ int clz64(unsigned long long m) {
@@ -837,11 +849,11 @@ __device__ __forceinline__ double positivity_tau(const double* qb, const double*
     double s3 = qb[3] + tau * d[3];
     double s4 = qb[4] + tau * d[4];
     double m2 = s1 * s1 + s2 * s2 + s3 * s3;
-    double ir = 1.0 / s0;
+    double ir = rcp64(s0);
     double f = gm1 * (s4 - 0.5 * m2 * ir) - eps;
     double md = s1 * d[1] + s2 * d[2] + s3 * d[3];
     double fp = gm1 * (d[4] - md * ir + 0.5 * m2 * d[0] * ir * ir);
-    double tn = tau - f / fp;
+    double tn = tau - f * rcp64(fp);
     if (!(tn >= 0.0)) tn = 0.0;
     if (tn > tau) tn = tau;
     double step = tau - tn;

@@ -38,7 +38,7 @@ namespace dg {
 template <int K>
 struct FusedCfg {
   static constexpr int Q = K + 1, Q2 = Q * Q, Q3 = Q2 * Q, N = nmodes(K), T = (K + 1) * (K + 2) / 2;
-  // plane tile: 8 x 8 cells at degree <= 2; 8 x 4 at degree 3, whose
+  // plane tile: 8 x 8 cells at degrees 1 and 2; 8 x 4 at degree 3, whose
   // Q^2 = 16 face points per face double the trace storage
   static constexpr int BX = 8, BY = K >= 3 ? 4 : 8, NC = BX * BY;
   static constexpr int THREADS = 5 * NC;  // one (cell, variable) per thread
@@ -65,7 +65,9 @@ struct FusedCfg {
   static constexpr int SMN = YL, SAB = YL + 5 * NC;
   static_assert(10 * NC <= 5 * Q2 * SZ, "screen buffers fit the left y traces");
   static constexpr size_t smem() { return sizeof(float) * (size_t)TOTAL; }
-  static constexpr int MINB = K >= 3 ? 3 : 2;  // CTAs per SM the register budget is sized for
+  // CTAs per SM the register budget is sized for (degree 1: 0.38 ms per stage at
+  // 100 x 90 x 84 with 2 or 3, 0.39 with 4)
+  static constexpr int MINB = K == 3 ? 3 : 2;
   static constexpr int NFACE = (SX + SY + NC) * Q2;
   // degree 3: the volume slices and the face points stay loops (unrolled,
   // the kernel outgrows the instruction cache: ncu showed instruction-fetch
@@ -760,6 +762,7 @@ __global__ void __launch_bounds__(FusedCfg<K>::THREADS, FusedCfg<K>::MINB) fused
     __syncthreads();
   }
   if (err) atomicOr(&a.ctrl->err, err);
+  if (a.stage > 0 && blockIdx.x == 0 && tid == 0) a.ctrl->n_deep = 0u;  // the limiter's second pass counts from 0
 }
 
 }  // namespace dg

@@ -49,12 +49,14 @@ cudaError_t fz_upload(const double* h64) {
 }
 
 // planes per z segment: the candidate with the fewest plane iterations per
-// SM over the waves of the grid (two tiles per SM on 152 SMs)
+// SM over the waves of the grid (MINB tiles per SM on 152 SMs); a segment takes
+// two iterations more than it has planes, so short ones only pay where the
+// chip is not full (16^3, degree 2: 24 us per stage with one plane, 59 with 4)
 int choose_lz(const Geo& g, long long columns) {
   const long long slots = 152LL * FC::MINB;
-  int best = 4;
+  int best = 1;
   long long best_cost = -1;
-  for (int lz : {4, 8, 16, 32, 64}) {
+  for (int lz : {1, 2, 4, 8, 16, 32, 64}) {
     const long long segs = (g.nz + lz - 1) / lz;
     const long long waves = (columns * segs + slots - 1) / slots;
     const long long cost = waves * (std::min(lz, g.nz) + 2);

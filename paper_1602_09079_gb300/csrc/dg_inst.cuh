@@ -98,8 +98,7 @@ cudaError_t upload(const double* h64, const float* h32) {
   h_tab64[dev] = static_cast<const double*>(p);
   if ((e = cudaGetSymbolAddress(&p, g_tab32)) != cudaSuccess) return e;
   h_tab32[dev] = static_cast<const float*>(p);
-  cudaError_t r = cudaFuncSetAttribute(limit_list_kernel<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)ListLim<KK>::smem());
+  cudaError_t r = cudaSuccess;
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(limit_screen_list_kernel<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)ListLim<KK>::smem());
@@ -217,16 +216,22 @@ cudaError_t volume_stage(int prec, bool force, const void* fh, const void* field
                : vol_t<double, MODE_STAGE, false>(ys, yf, fh, field, g, st, nullptr, ctrl, s);
 }
 
+// CTAs of a grid-stride kernel over a queue that holds at most nc cells
+inline unsigned limit_grid(long long nc, int per, unsigned most) {
+  const long long n = (nc + per - 1) / per;
+  return n < (long long)most ? (unsigned)n : most;
+}
+
 cudaError_t limit_list(double* y, const int* list, const unsigned* count, const Geo& g, Ctrl* ctrl, int count_queued,
                        float* yf, const double* y0, float* d, int* deep, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(&ctrl->n_deep, 0, sizeof(unsigned), s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   using LL = ListLim<KK>;
-  limit_screen_list_kernel<KK><<<152 * LL::MINB, LL::THREADS, LL::smem(), s>>>(
+  limit_screen_list_kernel<KK><<<limit_grid(g.nc, LL::THREADS, 152 * LL::MINB), LL::THREADS, LL::smem(), s>>>(
       y, list, count, tab_ptr<double>(), tab_ptr<float>(), g, ctrl, count_queued, deep);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  limit_list_kernel<KK><<<152 * LL::MINB, LL::THREADS, LL::smem(), s>>>(y, deep, &ctrl->n_deep, tab_ptr<double>(), g,
-                                                                       ctrl, yf, y0, d);
+  // a warp per cell
+  limit_list_kernel<KK><<<limit_grid(g.nc, LL::THREADS / 32, 152 * 4), LL::THREADS, LL::smem_deep(), s>>>(
+      y, deep, &ctrl->n_deep, tab_ptr<double>(), g, ctrl, yf, y0, d);
   return cudaGetLastError();
 }
 
@@ -240,8 +245,8 @@ cudaError_t limit(double* y, int8_t* flags, const Geo& g, Ctrl* ctrl, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t cfl(const double* y, const Geo& g, Ctrl* ctrl, cudaStream_t s) {
-  cfl_kernel<KK><<<grid1(g.nc, kCflThreads), kCflThreads, 0, s>>>(y, g, ctrl);
+cudaError_t cfl(const double* y, const Geo& g, Ctrl* ctrl, int slot, cudaStream_t s) {
+  cfl_kernel<KK><<<grid1(g.nc, kCflThreads), kCflThreads, 0, s>>>(y, g, ctrl, slot);
   return cudaGetLastError();
 }
 

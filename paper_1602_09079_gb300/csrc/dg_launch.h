@@ -26,7 +26,7 @@ struct Launchers {
   cudaError_t (*volume_rhs)(int prec, bool force, const double* y, const float* yf, const void* fh,
                             const void* field, const Geo& g, double* R, Ctrl* ctrl, cudaStream_t s);
   // SSP-RK3 stage combination + limiter screen: cells failing the screen are
-  // queued in list / ctrl->n_flag (ctrl->n_flag must be 0 on entry)
+  // queued in list / ctrl->n_flag (0 on entry)
   cudaError_t (*volume_stage)(int prec, bool force, const void* fh, const void* field, const Geo& g,
                               const double* ys, const double* y0, double* out, double a0, double b0,
                               double dt, int* list, float* yf, Ctrl* ctrl, cudaStream_t s);
@@ -42,7 +42,9 @@ struct Launchers {
   // screen[c] = 1 if cell c fails the limiter screen
   cudaError_t (*screen)(const double* y, uint8_t* screen, const Geo& g, cudaStream_t s);
   cudaError_t (*limit)(double* y, int8_t* flags, const Geo& g, Ctrl* ctrl, cudaStream_t s);
-  cudaError_t (*cfl)(const double* y, const Geo& g, Ctrl* ctrl, cudaStream_t s);
+  // slot: which of the control block's two maxima to use (zero on entry; the
+  // other one is cleared)
+  cudaError_t (*cfl)(const double* y, const Geo& g, Ctrl* ctrl, int slot, cudaStream_t s);
   // returns the number of partial sums written to part; cells failing the
   // limiter screen afterwards are queued in list / ctrl->n_flag (0 on entry)
   cudaError_t (*energy_reset)(int prec, double* y, const Geo& g, double c2g, double inv_rho0, double* part,
@@ -92,6 +94,7 @@ struct FusedLaunchers {
   cudaError_t (*run)(bool force, int flux, const Geo& g, FusedArgs& args, cudaStream_t s);
 };
 
+FusedLaunchers fused_launchers_k1();
 FusedLaunchers fused_launchers_k2();
 FusedLaunchers fused_launchers_k3();
 
