@@ -566,36 +566,81 @@ __device__ __forceinline__ void fx_project(const long long (&f)[K + 1], FxAcc (&
 }
 
 // ------------------------------------- FP64 reciprocal and square roots
-// One MUFU approximation of the significand (23 bits), then one third-order
-// Householder iteration (A. S. Householder, The Numerical Treatment of a
-// Single Nonlinear Equation, 1970) in FP64: 3 FP64 operations for 1/x, 5 for
-// 1/sqrt(x), within 2 units in the last place. Arguments near the ends of the
-// exponent range, zeros, infinities, NaNs (and x < 0 for the root) take the
-// library function.
+// One MUFU approximation y0 of the significand m (|1 - m y0| < 2^-21), then one
+// third-order Householder iteration (A. S. Householder, The Numerical Treatment
+// of a Single Nonlinear Equation, 1970), y0 (1 + r + r^2) with r = 1 - m y0 and
+// y0 (1 + r/2 + 3 r^2 / 8) with r = 1 - m y0^2, on the integer pipe: the exact
+// product gives r in units of 2^-82, the result has 60 bits before it is rounded
+// (within 0.51 units in the last place). In FP64 operations the iterations take
+// 3 and 5 of a pipe that retires two per clock and SM, which bounds the face
+// kernel (128^3, degree 2: 11.1 ms per stage so, now 9.15). Arguments near the ends of the exponent range, zeros,
+// infinities, NaNs (and x < 0 for the root) take the library function.
+
+// y0 (1 + c) rounded to a double's significand: y0 in units of 2^-30 (2^29 to
+// 2^30), c in units of 2^-60; e: biased exponent of the result for 0.5 <= y < 1,
+// less one
+__device__ __forceinline__ double root_finish(unsigned y0, long long c, unsigned e, unsigned sign) {
+  const long long p = (long long)((unsigned long long)y0 * (unsigned)c >> 30) + (long long)(int)(c >> 32) * (int)y0 * 4;
+  const unsigned long long y = ((unsigned long long)y0 << 30) + (unsigned long long)p;
+  const unsigned long long bits = ((unsigned long long)e << 52) + ((y + 64) >> 7);
+  return __longlong_as_double((long long)(bits | ((unsigned long long)sign << 32)));
+}
+
 __device__ __forceinline__ double rcp64(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int bx = bexp(hi);
   if ((unsigned)(bx - 64) > 1900u) return 1.0 / x;
-  const unsigned y = __float_as_uint(rcp_fast(__uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29))));
-  const unsigned e = (y >> 23) + (unsigned)(1919 - bx);  // (y - 127) - (bx - 1023) + 1023
-  const double y0 = __hiloint2double((int)((hi & 0x80000000u) | (e << 20) | ((y & 0x7fffffu) >> 3)), (int)(y << 29));
-  const double r = fma(-x, y0, 1.0);
-  return fma(y0, fma(r, r, r), y0);
+  const unsigned mh = (hi & 0xfffffu) | 0x100000u;  // significand, 53 bits
+  // (0.5, 1] in units of 2^-30
+  const unsigned y0 = (unsigned)(rcp_fast(__uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29))) * 0x1p30f);
+  // 1 - m y0 in units of 2^-82 (the product is 2^82 less this, modulo 2^64)
+  const long long r = -(long long)((unsigned long long)lo * y0 + ((unsigned long long)(mh * y0) << 32));
+  const int h = (int)(r >> 41);
+  return root_finish(y0, (r >> 22) + ((long long)h * h >> 22), (unsigned)(2044 - bx), hi & 0x80000000u);
 }
 __device__ __forceinline__ double rsqrt64(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int bx = (int)(hi >> 20);
   if ((unsigned)(bx - 64) > 1900u) return rsq(x);
-  const int odd = (bx - 1023) & 1, half = (bx - 1023 - odd) / 2;
-  const unsigned y = __float_as_uint(
-      rsqrt_fast(__uint_as_float(((127u + (unsigned)odd) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29))));
-  const double y0 = __hiloint2double((int)((((y >> 23) + (unsigned)(896 - half)) << 20) | ((y & 0x7fffffu) >> 3)),
-                                     (int)(y << 29));
-  const double r = fma(-x, y0 * y0, 1.0);
-  return fma(y0 * r, fma(r, 0.375, 0.5), y0);
+  const unsigned odd = (unsigned)(bx - 1023) & 1u;
+  const int half = (bx - 1023 - (int)odd) >> 1;
+  const unsigned f = ((127u + odd) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned y0 = (unsigned)(rsqrt_fast(__uint_as_float(f)) * 0x1p30f);
+  // significand in [1, 4), 54 bits
+  const unsigned long long m = (((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << odd;
+  const unsigned a0 = (unsigned)m, a1 = (unsigned)(m >> 32);
+  const unsigned k = y0 >> 6;  // y0's 24 bits: units of 2^-24, exact
+  const unsigned long long s = (unsigned long long)k * k;
+  const unsigned s0 = (unsigned)s, s1 = (unsigned)(s >> 32);
+  // 1 - m y0^2 in units of 2^-82, modulo 2^64
+  const unsigned long long t = (((unsigned long long)a0 * s0) >> 18) +
+                               (((unsigned long long)a0 * s1 + (unsigned long long)a1 * s0) << 14) +
+                               ((unsigned long long)(a1 * s1) << 46);
+  const long long r = -(long long)t;
+  const int h = (int)(r >> 41);
+  return root_finish(y0, (r >> 23) + ((long long)(3 * h) * h >> 25), (unsigned)(1021 - half), 0u);
 }
 // sqrt(max(x, 0))
 __device__ __forceinline__ double sqrt64(double x) { return __double2hiint(x) > 0 ? x * rsqrt64(x) : 0.0; }
+// x^(2/3) = z z^(-1/3) 2^(2q) for x = z 2^(3q), 1 <= z < 8: FP32 logarithm and
+// exponential (2^-20), then one third-order Householder iteration of z^(-1/3),
+// y (1 + e/3 + 2 e^2 / 9) with e = 1 - z y^3, in 7 FP64 operations (cbrt and a
+// square take about 30). x <= 0 and the ends of the exponent range take cbrt.
+__device__ __forceinline__ double pow_2_3(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int bx = (int)(hi >> 20);
+  if ((unsigned)(bx - 64) > 1900u) {
+    const double c = cbrt(x);
+    return c * c;
+  }
+  const int q = (bx - 1023 + 1200) / 3 - 400, s = bx - 1023 - 3 * q;
+  const double z = __hiloint2double((int)((hi & 0xfffffu) | ((unsigned)(1023 + s) << 20)), (int)lo);
+  const float f = __uint_as_float(((unsigned)(127 + s) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+  const double y = f32_to_f64_q(exp2f(log2f(f) * (-1.f / 3.f)));
+  const double e = fma(-(z * y), y * y, 1.0);
+  const double c = z * fma(y * e, fma(e, 2.0 / 9.0, 1.0 / 3.0), y);
+  return __hiloint2double(__double2hiint(c) + q * 0x200000, __double2loint(c));
+}
 // a < b in the total order of the bit patterns (integer pipe)
 __device__ __forceinline__ bool less64(double a, double b) {
   const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
@@ -604,8 +649,8 @@ __device__ __forceinline__ bool less64(double a, double b) {
 
 // HLLC flux of the face frame in FP64 (same algorithm as hllc_flux: Einfeldt
 // wave speeds, sound speed 0 at pressures <= 0, S* = 0 for a receding vacuum
-// interface), arranged for few FP64 operations, about 105 a point instead of
-// 190: the Roe sound speed from the average of the sides' c^2 and the velocity
+// interface), arranged for few FP64 operations, about 70 a point instead of
+// 190 (105 before the roots moved to the integer pipe): the Roe sound speed from the average of the sides' c^2 and the velocity
 // jump, c~^2 = <c^2> + (gamma - 1)/2 w (1 - w) |dv|^2 with the Roe weight w
 // (the same as through the total enthalpy); the flux of the star region as F(U*)
 // with the contact's speed and the star pressure (the jump conditions across

@@ -339,19 +339,19 @@ __device__ __forceinline__ unsigned face_f32_dir(const float* __restrict__ yf, f
 // tangential coefficients E, then along t2 and t1 to the values at the face's
 // Q^2 points, all in 64-bit fixed point (dg_common.cuh): both sides' values go
 // to shared memory in the face's frame. Then one numerical flux per face point
-// in FP64, which is what bounds the kernel (27 HLLC fluxes of about 105 FP64
-// operations per cell at degree 2, 2 operations per clock and SM). The fluxes go
+// in FP64, which with the integer work is what bounds the kernel (27 HLLC fluxes of
+// about 70 FP64 operations per cell at degree 2, 2 operations per clock and SM). The fluxes go
 // out as their T = (K+1)(K+2)/2 moments with the tangential modes,
 // [3][5][T][n_cells], once for the two cells that need them (MOMENTS; for the
 // dense volume_kernel the fluxes at the points, [3][5][Q^2][n_cells]). With FP64 contractions
-// and the 190-operation HLLC the kernel took 21.2 ms at 128^3, degree 2, now
-// 11.1 (the FP64 operations alone: 9.3).
+// and the 190-operation HLLC the kernel took 21.5 ms at 128^3, degree 2, now
+// 9.15 (the FP64 operations alone: 6.2).
 template <int K>
 struct FaceSF64 {
   static constexpr int C = 32, THREADS = 5 * C;
   static constexpr int Q2 = (K + 1) * (K + 1), T = (K + 1) * (K + 2) / 2;
-  // 4 CTAs per SM (96 registers) keep the FP64 pipe busier than 3 without
-  // spills: 11.1 against 12.6 ms at 128^3, degree 2
+  // CTAs per SM the register budget is sized for (128^3, degree 2: 9.15 ms with
+  // 4, 10.05 with 3, 9.04 with 5; 64^3, degree 3: 2.42, 2.49, 2.55)
   static constexpr int MINB = 4;
   // values [side][variable][point][cell]
   static constexpr size_t smem() { return sizeof(double) * 2 * 5 * Q2 * C; }
@@ -1965,7 +1965,9 @@ struct ResetConsts {
 // thread), then y and z per mode. Rows are padded to a multiple of 16 bytes
 // whose stride spreads the 8 rows of a quarter warp over all 32 banks. The
 // screen sums of rho and the momenta come from the coefficients the value
-// threads hold; those of E from the new modes.
+// threads hold; those of E from the new modes. FP64: values and projection in
+// fixed point (dg_common.cuh), a slice at a time, and x^(2/3) by one iteration:
+// 128^3, degree 2: 7.05 -> 2.23 ms.
 template <int K, typename T>
 struct ResetSF {
   static constexpr int C = 32;  // cells per block: one warp per variable
@@ -1996,7 +1998,7 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
   __shared__ double sEn[N * C];                // new energy modes [mode][cell]
   __shared__ double sM[5 * C];                 // means (old energy mean in row 4)
   __shared__ double sA[5 * C];                 // sum_l |w_il| max |phi_l|
-  __shared__ int sFin[5 * C];
+  __shared__ int sFin[(4 + Q) * C];            // finite flags; FP64: the slices' exponents
   clear_deep(ctrl);
   const long long nc = g.nc;
   const long long c0 = (long long)blockIdx.x * C;
@@ -2007,75 +2009,123 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
     const int i = tid / C, c = tid % C;  // warp = variable
     const long long cell = c0 + c;
     const bool in = cell < nc;
-    T w[N];
-    double mean = in ? y[(size_t)(i * N) * nc + cell] : (i == 0 ? 1.0 : 0.0);
-    if constexpr (sizeof(T) == 4) w[0] = f64_to_f32(mean);
-    else w[0] = mean;
+    if constexpr (sizeof(T) == 8) {
+      // FP64: sum-factorised in fixed point (dg_common.cuh), a slice at a time
+      using FT = FxTab<K>;
+      constexpr int T2 = (K + 1) * (K + 2) / 2, Q2 = Q * Q;
+      double w[N];
 #pragma unroll
-    for (int l = 1; l < N; ++l) {
-      if (!in) w[l] = T(0);
-      else if (from_shadow) w[l] = (T)yf[(size_t)(i * N + l) * nc + cell];
-      else w[l] = (T)y[(size_t)(i * N + l) * nc + cell];
-    }
-    sM[i * C + c] = mean;
-    if (tid < C) sM[4 * C + c] = in ? y[(size_t)(4 * N) * nc + cell] : 0.0;
-    // screen sums of this variable from the coefficients held (FP32: of the
-    // rounded coefficients, widened by a relative 1e-5, still an upper bound)
-    {
-      T sa = T(0);
-      bool fin = true;
+      for (int l = 0; l < N; ++l) w[l] = in ? y[(size_t)(i * N + l) * nc + cell] : (i == 0 && l == 0 ? 1.0 : 0.0);
+      sM[i * C + c] = w[0];
+      if (tid < C) sM[4 * C + c] = in ? y[(size_t)(4 * N) * nc + cell] : 0.0;
+      // screen sum (FP32 of the rounded coefficients, widened by a relative
+      // 1e-5, still an upper bound)
+      float sa = 0.f;
+      bool fin = finite64(w[0]);
 #pragma unroll
       for (int l = 1; l < N; ++l) {
-        T lm;
-        if constexpr (sizeof(T) == 4) lm = g.lim_vol ? c_tab32[TB::LMAXV + l] : c_tab32[TB::LMAX + l];
-        else lm = __ldg(tab + (g.lim_vol ? TB::LMAXV : TB::LMAX) + l);
-        sa += fabs(w[l]) * lm;
-        fin &= isfinite(w[l]);
+        sa = fmaf(abs_up(w[l]), c_tab32[(g.lim_vol ? TB::LMAXV : TB::LMAX) + l], sa);
+        fin &= finite64(w[l]);
       }
-      sA[i * C + c] = in ? (sizeof(T) == 4 ? (double)sa * (1.0 + 1e-5) : (double)sa) : 0.0;
-      sFin[i * C + c] = in ? (int)fin : 1;
-    }
-    // values at q = qx + Q (qy + Q qz): contract z, then y, then x with
-    // Pt_u(x_a) (sfc<T>(u Q + a))
-    T vals[Q3];
+      sA[i * C + c] = f32_to_f64_q(sa * (1.f + 1e-5f));
+      sFin[i * C + c] = (int)fin;
+      const int B = fx_bound<K>(w);
+      Fx x[N];
 #pragma unroll
-    for (int qz = 0; qz < Q; ++qz) {
-      T A1[(K + 1) * (K + 2) / 2];
+      for (int l = 0; l < N; ++l) x[l] = fx_split(fx_from(w[l], B));
+      T* out = sU + (i * C + c) * ROW;
+#pragma unroll 1
+      for (int qz = 0; qz < Q; ++qz) {
+        Fx A1[T2];
 #pragma unroll
-      for (int u = 0, j = 0; u <= K; ++u)
+        for (int u = 0, j = 0; u <= K; ++u)
 #pragma unroll
-        for (int v = 0; u + v <= K; ++v, ++j) {
-          T s = T(0);
+          for (int v = 0; u + v <= K; ++v, ++j) {
+            FxAcc s{0, 0};
 #pragma unroll
-          for (int ww = 0; u + v + ww <= K; ++ww) s += w[mode_index(u, v, ww)] * sfc<T>(ww * Q + qz);
-          A1[j] = s;
-        }
+            for (int ww = 1; u + v + ww <= K; ++ww) fx_madt(s, x[mode_index(u, v, ww)], FT::P + ww * Q + qz);
+            const long long x0 = fx_join(x[mode_index(u, v, 0)]);
+            A1[j] = fx_split(u + v < K ? fx_val(s) + x0 : x0);
+          }
+        Fx A2[Q][K + 1];
+        fx_rows<K, 0>(A1, A2);
 #pragma unroll
-      for (int qy = 0; qy < Q; ++qy) {
-        T A2[K + 1];
+        for (int qy = 0; qy < Q; ++qy) {
+          long long v[Q];
+          fx_values<K, K + 1>(A2[qy], v);
 #pragma unroll
-        for (int u = 0, j = 0; u <= K; ++u) {
-          T s = T(0);
-#pragma unroll
-          for (int v = 0; u + v <= K; ++v, ++j) s += A1[j] * sfc<T>(v * Q + qy);
-          A2[u] = s;
-        }
-#pragma unroll
-        for (int qx = 0; qx < Q; ++qx) {
-          T s = T(0);
-#pragma unroll
-          for (int u = 0; u <= K; ++u) s += A2[u] * sfc<T>(u * Q + qx);
-          vals[qx + Q * (qy + Q * qz)] = s;
+          for (int qx = 0; qx < Q; ++qx)
+            out[qz * Q2 + qy * Q + qx] = B < kFxHuge ? fx_to_double(v[qx], B) : __longlong_as_double(0x7ff8000000000000LL);
         }
       }
-    }
-    Vec* out = reinterpret_cast<Vec*>(sU + (i * C + c) * ROW);
+    } else {
+      T w[N];
+      double mean = in ? y[(size_t)(i * N) * nc + cell] : (i == 0 ? 1.0 : 0.0);
+      w[0] = f64_to_f32(mean);
 #pragma unroll
-    for (int k = 0; k < ROW / V; ++k) {
-      Vec t;
+      for (int l = 1; l < N; ++l) {
+        if (!in) w[l] = T(0);
+        else if (from_shadow) w[l] = (T)yf[(size_t)(i * N + l) * nc + cell];
+        else w[l] = (T)y[(size_t)(i * N + l) * nc + cell];
+      }
+      sM[i * C + c] = mean;
+      if (tid < C) sM[4 * C + c] = in ? y[(size_t)(4 * N) * nc + cell] : 0.0;
+      // screen sums of this variable from the coefficients held (FP32: of the
+      // rounded coefficients, widened by a relative 1e-5, still an upper bound)
+      {
+        T sa = T(0);
+        bool fin = true;
 #pragma unroll
-      for (int e = 0; e < V; ++e) t.v[e] = k * V + e < Q3 ? vals[k * V + e] : T(0);
-      out[k] = t;
+        for (int l = 1; l < N; ++l) {
+          const T lm = g.lim_vol ? c_tab32[TB::LMAXV + l] : c_tab32[TB::LMAX + l];
+          sa += fabs(w[l]) * lm;
+          fin &= isfinite(w[l]);
+        }
+        sA[i * C + c] = in ? (double)sa * (1.0 + 1e-5) : 0.0;
+        sFin[i * C + c] = in ? (int)fin : 1;
+      }
+      // values at q = qx + Q (qy + Q qz): contract z, then y, then x with
+      // Pt_u(x_a) (sfc<T>(u Q + a))
+      T vals[Q3];
+#pragma unroll
+      for (int qz = 0; qz < Q; ++qz) {
+        T A1[(K + 1) * (K + 2) / 2];
+#pragma unroll
+        for (int u = 0, j = 0; u <= K; ++u)
+#pragma unroll
+          for (int v = 0; u + v <= K; ++v, ++j) {
+            T s = T(0);
+#pragma unroll
+            for (int ww = 0; u + v + ww <= K; ++ww) s += w[mode_index(u, v, ww)] * sfc<T>(ww * Q + qz);
+            A1[j] = s;
+          }
+#pragma unroll
+        for (int qy = 0; qy < Q; ++qy) {
+          T A2[K + 1];
+#pragma unroll
+          for (int u = 0, j = 0; u <= K; ++u) {
+            T s = T(0);
+#pragma unroll
+            for (int v = 0; u + v <= K; ++v, ++j) s += A1[j] * sfc<T>(v * Q + qy);
+            A2[u] = s;
+          }
+#pragma unroll
+          for (int qx = 0; qx < Q; ++qx) {
+            T s = T(0);
+#pragma unroll
+            for (int u = 0; u <= K; ++u) s += A2[u] * sfc<T>(u * Q + qx);
+            vals[qx + Q * (qy + Q * qz)] = s;
+          }
+        }
+      }
+      Vec* out = reinterpret_cast<Vec*>(sU + (i * C + c) * ROW);
+#pragma unroll
+      for (int k = 0; k < ROW / V; ++k) {
+        Vec t;
+#pragma unroll
+        for (int e = 0; e < V; ++e) t.v[e] = k * V + e < Q3 ? vals[k * V + e] : T(0);
+        out[k] = t;
+      }
     }
   }
   __syncthreads();
@@ -2090,13 +2140,18 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
     // gamma = 5/3 (gamma - 1 within 1e-15 of 2/3): x^(2/3) as cbrt(x)^2
     const T x = r * tir0;
     T xg;
-    if (two_thirds) {
-      const T cx = cbrt(x);
-      xg = cx * cx;
+    if constexpr (sizeof(T) == 8) {
+      xg = two_thirds ? pow_2_3(x) : pow(x, gm1);
+      sE[c * ROW + q] = fma(0.5 * fma(m1, m1, fma(m2, m2, m3 * m3)), rcp64(r), r * (tc2g * xg));
     } else {
-      xg = pow(x, gm1);
+      if (two_thirds) {
+        const T cx = cbrt(x);
+        xg = cx * cx;
+      } else {
+        xg = pow(x, gm1);
+      }
+      sE[c * ROW + q] = T(0.5) * (m1 * m1 + m2 * m2 + m3 * m3) / r + r * (tc2g * xg);
     }
-    sE[c * ROW + q] = T(0.5) * (m1 * m1 + m2 * m2 + m3 * m3) / r + r * (tc2g * xg);
   }
   __syncthreads();
   // --------------------------------------------------- projection of E
@@ -2104,45 +2159,103 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
   // qz, qy) per thread, into the dead point-value rows), then every mode
   // (u, v, w) as sum_qz Pt_w w_qz sum_qy Pt_v w_qy G[(qz, qy)][u] (one
   // (cell, mode) per thread); Pt w from the 1D tables (sfc<T>(KQ + u Q + a))
-  constexpr int KQ = (K + 1) * Q, GROW = Q * Q * (K + 1);
-  T* sG = sU;  // [cell][(qz Q + qy) (K + 1) + u]
-  for (int it = tid; it < Q * Q * C; it += RS::THREADS) {
-    const int c = it / (Q * Q), r = it - c * (Q * Q);  // r = qz Q + qy
-    const T* e = sE + c * ROW + r * Q;
-    T ev[Q];
+  if constexpr (sizeof(T) == 8) {
+    // FP64: one (cell, slice) per thread in fixed point, the slices summed per
+    // mode
+    using FT = FxTab<K>;
+    long long* sAcc = reinterpret_cast<long long*>(smem_raw);  // [slice][mode][cell]
+    int* sExp = sFin + 4 * C;                                  // [slice][cell]
+    if (tid < Q * C) {
+      const int qz = tid / C, c = tid % C;
+      const T* e = sE + c * ROW + qz * Q * Q;
+      unsigned mx = 0;
 #pragma unroll
-    for (int qx = 0; qx < Q; ++qx) ev[qx] = e[qx];
+      for (int q = 0; q < Q * Q; ++q) mx = max(mx, (unsigned)__double2hiint(e[q]) & 0x7fffffffu);
+      const int A = max(kFxTiny, bexp(mx) + 1);
+      long long G[K + 1][Q];  // [u][qy]
 #pragma unroll
-    for (int u = 0; u <= K; ++u) {
-      T s = T(0);
+      for (int qy = 0; qy < Q; ++qy) {
+        long long v[Q];
+        FxAcc r[K + 1];
 #pragma unroll
-      for (int qx = 0; qx < Q; ++qx) s += ev[qx] * sfc<T>(KQ + u * Q + qx);
-      sG[c * GROW + r * (K + 1) + u] = s;
+        for (int q = 0; q < Q; ++q) {
+          v[q] = fx_from(e[qy * Q + q], A);
+          r[q] = {0, 0};
+        }
+        fx_project<K, false>(v, r);
+#pragma unroll
+        for (int u = 0; u <= K; ++u) G[u][qy] = fx_val(r[u]);
+      }
+#pragma unroll
+      for (int u = 0; u <= K; ++u) {
+        FxAcc h[K + 1];
+#pragma unroll
+        for (int v = 0; v <= K; ++v) h[v] = {0, 0};
+        fx_project<K, false>(G[u], h);
+#pragma unroll
+        for (int v = 0; u + v <= K; ++v) {
+          const Fx hx = fx_split(fx_val(h[v]));
+#pragma unroll
+          for (int ww = 0; u + v + ww <= K; ++ww) {
+            FxAcc t{0, 0};
+            fx_mad(t, hx, c_fx[FT::W + ww * Q + qz][0], c_fx[FT::W + ww * Q + qz][1]);
+            sAcc[(qz * N + mode_index(u, v, ww)) * C + c] = fx_val(t);
+          }
+        }
+      }
+      sExp[qz * C + c] = bexp(mx) < kFxHuge ? A : 2 * kFxHuge;
     }
-  }
-  __syncthreads();
-  for (int it = tid; it < N * C; it += RS::THREADS) {
-    const int l = it / C, c = it - l * C;  // a warp: one mode of 32 cells
-    int u, v, ww;
-    mode_uvw(l, u, v, ww);
-    T pv[Q], pz[Q];
+    __syncthreads();
+    for (int it = tid; it < N * C; it += RS::THREADS) {
+      const int l = it / C, c = it - l * C;
+      int A = 0;
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      pv[q] = sfc<T>(KQ + v * Q + q);
-      pz[q] = sfc<T>(KQ + ww * Q + q);
+      for (int z = 0; z < Q; ++z) A = max(A, sExp[z * C + c]);
+      long long t = 0;
+#pragma unroll
+      for (int z = 0; z < Q; ++z) t += sAcc[(z * N + l) * C + c] >> min(A - sExp[z * C + c], 63);
+      sEn[it] = A < kFxHuge ? fx_to_double(t, A) : __longlong_as_double(0x7ff8000000000000LL);
     }
-    const T* gc = sG + c * GROW + u;
-    T acc = T(0);
+  } else {
+    constexpr int KQ = (K + 1) * Q, GROW = Q * Q * (K + 1);
+    T* sG = sU;  // [cell][(qz Q + qy) (K + 1) + u]
+    for (int it = tid; it < Q * Q * C; it += RS::THREADS) {
+      const int c = it / (Q * Q), r = it - c * (Q * Q);  // r = qz Q + qy
+      const T* e = sE + c * ROW + r * Q;
+      T ev[Q];
 #pragma unroll
-    for (int qz = 0; qz < Q; ++qz) {
-      T h = T(0);
+      for (int qx = 0; qx < Q; ++qx) ev[qx] = e[qx];
 #pragma unroll
-      for (int qy = 0; qy < Q; ++qy) h += gc[(qz * Q + qy) * (K + 1)] * pv[qy];
-      acc += h * pz[qz];
+      for (int u = 0; u <= K; ++u) {
+        T s = T(0);
+#pragma unroll
+        for (int qx = 0; qx < Q; ++qx) s += ev[qx] * sfc<T>(KQ + u * Q + qx);
+        sG[c * GROW + r * (K + 1) + u] = s;
+      }
     }
-    acc *= T(0.125);  // the reference cell's volume 8: w_l = 1/8 sum_q E phi_l w_q
-    if constexpr (sizeof(T) == 4) sEn[l * C + c] = f32_to_f64(acc);
-    else sEn[l * C + c] = acc;
+    __syncthreads();
+    for (int it = tid; it < N * C; it += RS::THREADS) {
+      const int l = it / C, c = it - l * C;  // a warp: one mode of 32 cells
+      int u, v, ww;
+      mode_uvw(l, u, v, ww);
+      T pv[Q], pz[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        pv[q] = sfc<T>(KQ + v * Q + q);
+        pz[q] = sfc<T>(KQ + ww * Q + q);
+      }
+      const T* gc = sG + c * GROW + u;
+      T acc = T(0);
+#pragma unroll
+      for (int qz = 0; qz < Q; ++qz) {
+        T h = T(0);
+#pragma unroll
+        for (int qy = 0; qy < Q; ++qy) h += gc[(qz * Q + qy) * (K + 1)] * pv[qy];
+        acc += h * pz[qz];
+      }
+      acc *= T(0.125);  // the reference cell's volume 8: w_l = 1/8 sum_q E phi_l w_q
+      sEn[l * C + c] = f32_to_f64(acc);
+    }
   }
   __syncthreads();
   // ------------------------------- screen of the reset state, dissipation
@@ -2150,25 +2263,14 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
   if (tid < C && c0 + tid < nc) {
     const int c = tid;
     const long long cell = c0 + c;
-    double ae = 0.0;
-    bool fin = isfinite(sEn[c]);
-    if constexpr (sizeof(T) == 4) {
-      float sf = 0.f;
+    bool fin = finite64(sEn[c]);
+    float sf = 0.f;
 #pragma unroll
-      for (int l = 1; l < N; ++l) {
-        const float v = f64_to_f32(sEn[l * C + c]);
-        sf += fabsf(v) * (g.lim_vol ? c_tab32[TB::LMAXV + l] : c_tab32[TB::LMAX + l]);
-        fin &= isfinite(v);
-      }
-      ae = (double)sf * (1.0 + 1e-5);
-    } else {
-#pragma unroll
-      for (int l = 1; l < N; ++l) {
-        const double v = sEn[l * C + c];
-        ae += fabs(v) * __ldg(tab + (g.lim_vol ? TB::LMAXV : TB::LMAX) + l);
-        fin &= isfinite(v);
-      }
+    for (int l = 1; l < N; ++l) {
+      sf = fmaf(abs_up(sEn[l * C + c]), g.lim_vol ? c_tab32[TB::LMAXV + l] : c_tab32[TB::LMAX + l], sf);
+      fin &= finite64(sEn[l * C + c]);
     }
+    const double ae = (double)sf * (1.0 + 1e-5);
     const double r = sM[c], m1 = sM[C + c], m2 = sM[2 * C + c], m3 = sM[3 * C + c];
     const double kin = 0.5 * (m1 * m1 + m2 * m2 + m3 * m3) / r;
     diss = (sM[4 * C + c] - kin) - (sEn[c] - kin);
