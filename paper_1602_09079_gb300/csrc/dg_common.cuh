@@ -7,6 +7,16 @@
 
 namespace dg {
 
+// First statement of every kernel that is launched with programmatic stream
+// serialisation (launch_after): the kernel may be set up while its predecessor
+// in the stream still runs; this waits until that one has completed and its
+// writes are visible, before anything is read or written.
+__device__ __forceinline__ void stream_wait() {
+#ifdef __CUDA_ARCH__
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+#endif
+}
+
 // ------------------------------------------------------------- sizes
 __host__ __device__ constexpr int nmodes(int k) { return (k + 1) * (k + 2) * (k + 3) / 6; }
 __host__ __device__ constexpr int gll_m(int k) { return k <= 1 ? 2 : 3; }
@@ -40,6 +50,31 @@ __device__ __forceinline__ void mode_uvw(int l, int& u, int& v, int& w) {
   v = D - u - r;
   w = D - u - v;
 }
+
+// 8 x 8 matrices of 16-bit elements from shared memory in the fragment layout of
+// mma.sync (PTX ldmatrix): lane l gives the address of row l % 8 of matrix l / 8;
+// lane (g, t) = (l / 4, l % 4) receives elements [g][2t], [g][2t + 1] of every
+// matrix, transposed [2t][g], [2t + 1][g]. Rows are 16-byte aligned.
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p))
+               : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p))
+               : "memory");
+}
+__device__ __forceinline__ void ldsm2_t(uint32_t (&r)[2], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1])
+               : "r"((uint32_t)__cvta_generic_to_shared(p))
+               : "memory");
+}
+#endif
 
 // Per-degree basis/quadrature tables (Sect. 2.2-2.5), all values at the
 // method's point sets, offsets in elements. Weights are folded in so the
@@ -720,6 +755,16 @@ __device__ __forceinline__ void hllc64_x(const double* UL, const double* UR, dou
 // non-finite pressure.
 constexpr int kExactIters = 50;
 
+// x^z for x > 0 and the small exponent z = (gamma - 1) / (2 gamma) < 1/2. FP32:
+// through log2f and exp2f; their error enters the jump x^z - 1 with at most
+// max_t t 2^-t = 0.53 of an ulp of 1 for x <= 1, less than powf's own rounding
+// there, at a third of its instructions.
+template <typename T>
+__device__ __forceinline__ T pow_z(T x, T z) {
+  if constexpr (sizeof(T) == 4) return exp2f(z * log2f(x));
+  else return pow(x, z);
+}
+
 template <typename T>
 struct ExactSide {
   T rho, u, p, c;
@@ -740,11 +785,18 @@ struct ExactSide {
   // f_K(ps) and its derivative; z = (gamma - 1) / (2 gamma)
   __device__ __forceinline__ void jump(T ps, T z, T gamma, T& f, T& df) const {
     if (ps > p) {
-      const T q = sqrt(A / (ps + B));
-      f = (ps - p) * q;
-      df = q * (T(1) - T(0.5) * (ps - p) / (ps + B));
+      if constexpr (sizeof(T) == 4) {
+        const T i = T(1) / (ps + B);
+        const T q = sqrt(A * i);
+        f = (ps - p) * q;
+        df = q * (T(1) - T(0.5) * (ps - p) * i);
+      } else {
+        const T q = sqrt(A / (ps + B));
+        f = (ps - p) * q;
+        df = q * (T(1) - T(0.5) * (ps - p) / (ps + B));
+      }
     } else {
-      const T r = pow(ps / p, z);
+      const T r = pow_z(ps / p, z);
       f = crf * (r - T(1));
       df = c * r / (gamma * ps);
     }
@@ -843,7 +895,7 @@ __device__ __forceinline__ unsigned exact_flux(int d, const T* UL, const T* UR, 
         W[0] = K.rho * (ratio + g6) / (g6 * ratio + T(1)); W[1] = us; W[2] = ps;
       }
     } else {
-      const T head = K.u - sg * K.c, tail = us - sg * K.c * pow(ratio, z);
+      const T head = K.u - sg * K.c, tail = us - sg * K.c * pow_z(ratio, z);
       if (sg * head >= T(0)) {
         W[0] = K.rho; W[1] = K.u; W[2] = K.p;
       } else if (sg * tail < T(0)) {

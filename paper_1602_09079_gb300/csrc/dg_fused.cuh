@@ -296,6 +296,7 @@ __device__ __forceinline__ void fz_apply(const float (&Hl)[(K + 1) * (K + 2) / 2
 
 template <int K, bool FORCE, int FLUX>
 __global__ void __launch_bounds__(FusedCfg<K>::THREADS, FusedCfg<K>::MINB) fused_f32_kernel(Geo g, FusedArgs a) {
+  stream_wait();
   using CF = FusedCfg<K>;
   using TB = FzTab<K>;
   constexpr int Q = CF::Q, Q2 = CF::Q2, Q3 = CF::Q3, N = CF::N, T = CF::T;

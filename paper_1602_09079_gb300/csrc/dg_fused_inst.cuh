@@ -3,6 +3,7 @@
 #pragma once
 #include "dg_fused.cuh"
 #include "dg_launch.h"
+#include "dg_stream_launch.h"
 
 #include <algorithm>
 
@@ -78,14 +79,12 @@ cudaError_t fz_run(bool force, int flux, const Geo& g, FusedArgs& a, cudaStream_
   const long long grid = columns * ((g.nz + a.lz - 1) / a.lz);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   const unsigned nb = (unsigned)grid;
-  if (flux == 1) {
-    if (force) fused_f32_kernel<FK, true, 1><<<nb, FC::THREADS, FC::smem(), s>>>(g, a);
-    else fused_f32_kernel<FK, false, 1><<<nb, FC::THREADS, FC::smem(), s>>>(g, a);
-  } else {
-    if (force) fused_f32_kernel<FK, true, 0><<<nb, FC::THREADS, FC::smem(), s>>>(g, a);
-    else fused_f32_kernel<FK, false, 0><<<nb, FC::THREADS, FC::smem(), s>>>(g, a);
-  }
-  return cudaGetLastError();
+  const size_t sm = FC::smem();
+  if (flux == 1)
+    return force ? launch_after(fused_f32_kernel<FK, true, 1>, nb, FC::THREADS, sm, s, g, a)
+                 : launch_after(fused_f32_kernel<FK, false, 1>, nb, FC::THREADS, sm, s, g, a);
+  return force ? launch_after(fused_f32_kernel<FK, true, 0>, nb, FC::THREADS, sm, s, g, a)
+               : launch_after(fused_f32_kernel<FK, false, 0>, nb, FC::THREADS, sm, s, g, a);
 }
 
 }  // namespace

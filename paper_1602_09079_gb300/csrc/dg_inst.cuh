@@ -5,6 +5,7 @@
 
 #include "dg_kernels.cuh"
 #include "dg_launch.h"
+#include "dg_stream_launch.h"
 
 #ifndef DG_K
 #error "define DG_K before including dg_inst.cuh"
@@ -134,9 +135,8 @@ cudaError_t face64(const double* y, void* fh, const Geo& g, Ctrl* ctrl, cudaStre
   // chip's CTA slots (6 x 8 x 7 at degree 2: 21 us instead of 52; from there on
   // the second load of a tile's coefficients costs what the waves gain)
   const unsigned tiles = grid1(g.nc, 32);
-  face_sf64_kernel<KK, FLUX, kSumFact><<<dim3(tiles, tiles * 2 < 152u * CF::MINB ? 3 : 1), CF::THREADS, CF::smem(), s>>>(
-      y, static_cast<double*>(fh), g, ctrl);
-  return cudaGetLastError();
+  return launch_after(face_sf64_kernel<KK, FLUX, kSumFact>, dim3(tiles, tiles * 2 < 152u * CF::MINB ? 3 : 1),
+      CF::THREADS, CF::smem(), s, y, static_cast<double*>(fh), g, ctrl);
 }
 
 // FP32 path: the face kernel (constant-bank tables) reads the FP32 shadow at
@@ -146,8 +146,9 @@ cudaError_t face64(const double* y, void* fh, const Geo& g, Ctrl* ctrl, cudaStre
 template <int FLUX>
 cudaError_t face_f(int prec, const double* y, const float* yf, void* fh, const Geo& g, Ctrl* ctrl, cudaStream_t s) {
   if (prec) {  // FP32 path: sum-factorised traces of the FP32 shadow
-    face_flux_f32_kernel<KK, FLUX><<<grid1(g.nc, 32), 96, 0, s>>>(yf, static_cast<float*>(fh), g, ctrl);
-    return cudaGetLastError();
+    return launch_after(face_flux_f32_kernel<KK, FLUX>, grid1(g.nc, 32), 96, 0, s, yf, static_cast<float*>(fh), g,
+        ctrl);
+
   }
   return face64<FLUX>(y, fh, g, ctrl, s);
 }
@@ -161,30 +162,28 @@ template <int MODE, bool FORCE>
 cudaError_t vol_f32(const float* yf, const void* fh, const void* field, const Geo& g, StageArgs st, double* R,
                     Ctrl* ctrl, cudaStream_t s) {
   using CF = VolF32<KK>;
-  volume_f32_kernel<KK, MODE, FORCE><<<grid1(g.nc, CF::C), CF::THREADS, CF::smem(FORCE), s>>>(
-      yf, static_cast<const float*>(fh), static_cast<const float*>(field), tab_ptr<double>(), g, st, R, ctrl);
-  return cudaGetLastError();
+  return launch_after(volume_f32_kernel<KK, MODE, FORCE>, grid1(g.nc, CF::C), CF::THREADS, CF::smem(FORCE), s, yf,
+      static_cast<const float*>(fh), static_cast<const float*>(field), tab_ptr<double>(), g, st, R, ctrl);
 }
 
 template <typename T, int MODE, bool FORCE>
 cudaError_t vol_t(const double* y, const float* yf, const void* fh, const void* field, const Geo& g, StageArgs st,
                   double* R, Ctrl* ctrl, cudaStream_t s) {
+  cudaError_t e;
   if constexpr (kSumFact && sizeof(T) == 8) {
     using CF = VolSF<KK, T>;
-    volume_sf_kernel<KK, T, MODE, FORCE><<<grid1(g.nc, CF::C), kThreads, CF::smem(), s>>>(
-        y, yf, static_cast<const T*>(fh), static_cast<const T*>(field), tab_ptr<T>(), tab_ptr<double>(), g, st, R,
-        ctrl);
+    e = launch_after(volume_sf_kernel<KK, T, MODE, FORCE>, grid1(g.nc, CF::C), kThreads, CF::smem(), s, y, yf,
+        static_cast<const T*>(fh), static_cast<const T*>(field), tab_ptr<T>(), tab_ptr<double>(), g, st, R, ctrl);
   } else if constexpr (kSumFact) {
     using CF = VolSF<KK, T>;
-    volume_sfb_kernel<KK, T, MODE, FORCE><<<grid1(g.nc, CF::C), kThreads, CF::smem(), s>>>(
-        y, yf, static_cast<const T*>(fh), static_cast<const T*>(field), tab_ptr<T>(), tab_ptr<double>(), g, st, R,
-        ctrl);
+    e = launch_after(volume_sfb_kernel<KK, T, MODE, FORCE>, grid1(g.nc, CF::C), kThreads, CF::smem(), s, y, yf,
+        static_cast<const T*>(fh), static_cast<const T*>(field), tab_ptr<T>(), tab_ptr<double>(), g, st, R, ctrl);
   } else {
     using CF = VolCfg<KK, T>;
-    volume_kernel<KK, T, MODE, FORCE><<<grid1(g.nc, CF::C), kThreads, CF::smem(FORCE), s>>>(
-        y, static_cast<const T*>(fh), static_cast<const T*>(field), tab_ptr<T>(), tab_ptr<double>(), g, st, R, ctrl);
+    e = launch_after(volume_kernel<KK, T, MODE, FORCE>, grid1(g.nc, CF::C), kThreads, CF::smem(FORCE), s, y,
+        static_cast<const T*>(fh), static_cast<const T*>(field), tab_ptr<T>(), tab_ptr<double>(), g, st, R, ctrl);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t volume_rhs(int prec, bool force, const double* y, const float* yf, const void* fh, const void* field,
@@ -226,13 +225,13 @@ cudaError_t limit_list(double* y, const int* list, const unsigned* count, const 
                        float* yf, const double* y0, float* d, int* deep, cudaStream_t s) {
   cudaError_t e;
   using LL = ListLim<KK>;
-  limit_screen_list_kernel<KK><<<limit_grid(g.nc, LL::THREADS, 152 * LL::MINB), LL::THREADS, LL::smem(), s>>>(
-      y, list, count, tab_ptr<double>(), tab_ptr<float>(), g, ctrl, count_queued, deep);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_after(limit_screen_list_kernel<KK>, limit_grid(g.nc, LL::THREADS, 152 * LL::MINB), LL::THREADS,
+      LL::smem(), s, y, list, count, tab_ptr<double>(), tab_ptr<float>(), g, ctrl, count_queued, deep)) !=
+      cudaSuccess) return e;
+
   // a warp per cell
-  limit_list_kernel<KK><<<limit_grid(g.nc, LL::THREADS / 32, 152 * 4), LL::THREADS, LL::smem_deep(), s>>>(
-      y, deep, &ctrl->n_deep, tab_ptr<double>(), g, ctrl, yf, y0, d);
-  return cudaGetLastError();
+  return launch_after(limit_list_kernel<KK>, limit_grid(g.nc, LL::THREADS / 32, 152 * 4), LL::THREADS,
+      LL::smem_deep(), s, y, deep, &ctrl->n_deep, tab_ptr<double>(), g, ctrl, yf, y0, d);
 }
 
 cudaError_t screen(const double* y, uint8_t* scr, const Geo& g, cudaStream_t s) {
@@ -246,8 +245,7 @@ cudaError_t limit(double* y, int8_t* flags, const Geo& g, Ctrl* ctrl, cudaStream
 }
 
 cudaError_t cfl(const double* y, const Geo& g, Ctrl* ctrl, int slot, cudaStream_t s) {
-  cfl_kernel<KK><<<grid1(g.nc, kCflThreads), kCflThreads, 0, s>>>(y, g, ctrl, slot);
-  return cudaGetLastError();
+  return launch_after(cfl_kernel<KK>, grid1(g.nc, kCflThreads), kCflThreads, 0, s, y, g, ctrl, slot);
 }
 
 template <typename T>
@@ -261,8 +259,8 @@ cudaError_t reset_t(double* y, const Geo& g, double c2g, double inv_rho0, double
   rc.inv_rho0 = (T)inv_rho0;
   rc.gm1 = (T)(g.gamma - 1.0);
   rc.two_thirds = std::fabs(g.gamma - 1.0 - 2.0 / 3.0) < 1e-15 ? 1 : 0;
-  energy_reset_sf_kernel<KK, T><<<nb, RS::THREADS, RS::smem(), s>>>(y, tab_ptr<T>(), g, rc, part, list, ctrl, yf);
-  return cudaGetLastError();
+  return launch_after(energy_reset_sf_kernel<KK, T>, nb, RS::THREADS, RS::smem(), s, y, tab_ptr<T>(), g, rc, part,
+      list, ctrl, yf);
 }
 
 cudaError_t diagnostics(int prec, const double* y, const void* field, int force, const Geo& g, double* part, int nb,
@@ -299,7 +297,6 @@ cudaError_t forcing_field(int prec, void* field, const double* modes, int n, con
                           cudaStream_t s) {
   return prec ? field_t<float>(field, modes, n, g, L, s) : field_t<double>(field, modes, n, g, L, s);
 }
-
 }  // namespace
 
 #define DG_PASTE2(a, b) a##b
@@ -324,5 +321,4 @@ Launchers DG_PASTE(launchers_k, DG_K)() {
   L.table_size = TB::SIZE;
   return L;
 }
-
 }  // namespace dg

@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(kThreads) volume_kernel(const double* __restri
                                                           const T* __restrict__ field, const T* __restrict__ tab,
                                                           const double* __restrict__ tab64, Geo g, StageArgs st,
                                                           double* __restrict__ R, Ctrl* ctrl) {
+  stream_wait();
   using TB = Tab<K>;
   using CF = VolCfg<K, T>;
   constexpr int N = TB::N, Q2 = TB::Q2, Q3 = TB::Q3, C = CF::C;
@@ -345,25 +346,34 @@ __device__ __forceinline__ unsigned face_f32_dir(const float* __restrict__ yf, f
 // [3][5][T][n_cells], once for the two cells that need them (MOMENTS; for the
 // dense volume_kernel the fluxes at the points, [3][5][Q^2][n_cells]). With FP64 contractions
 // and the 190-operation HLLC the kernel took 21.5 ms at 128^3, degree 2, now
-// 9.15 (the FP64 operations alone: 6.2).
+// 8.74 (the FP64 operations alone: 6.2).
 template <int K>
 struct FaceSF64 {
   static constexpr int C = 32, THREADS = 5 * C;
   static constexpr int Q2 = (K + 1) * (K + 1), T = (K + 1) * (K + 2) / 2;
-  // CTAs per SM the register budget is sized for (128^3, degree 2: 9.15 ms with
-  // 4, 10.05 with 3, 9.04 with 5; 64^3, degree 3: 2.42, 2.49, 2.55)
-  static constexpr int MINB = 4;
+  // CTAs per SM the register budget is sized for (128^3, degree 2: 8.74 ms with
+  // 5, 8.85 with 4; 64^3, degree 3: 2.36, 2.41)
+  static constexpr int MINB = 5;
   // values [side][variable][point][cell]
   static constexpr size_t smem() { return sizeof(double) * 2 * 5 * Q2 * C; }
 };
 
+// index of the mode with the exponents (e, a, b) along (normal, tangential 1,
+// tangential 2) of a face normal to d, by the index of (e, a, b) as (u, v, w)
+static __constant__ unsigned char c_face_order[3][20] = {
+    {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19},
+    {0, 2, 1, 3, 7, 5, 8, 4, 6, 9, 16, 13, 17, 11, 14, 18, 10, 12, 15, 19},
+    {0, 3, 1, 2, 9, 6, 8, 4, 5, 7, 19, 15, 18, 12, 14, 17, 10, 11, 13, 16}};
+
 // coefficients of one (cell, variable) in fixed point, exponent B; row stride nc
+// (order: the modes' order along the face's axes)
 template <int K>
-__device__ __forceinline__ void fx_load(const double* __restrict__ p, size_t nc, Fx (&x)[nmodes(K)], int& B) {
+__device__ __forceinline__ void fx_load(const double* __restrict__ p, size_t nc, Fx (&x)[nmodes(K)], int& B,
+                                        const unsigned char* order = nullptr) {
   constexpr int N = nmodes(K);
   double w[N];
 #pragma unroll
-  for (int l = 0; l < N; ++l) w[l] = __ldg(p + (size_t)l * nc);
+  for (int l = 0; l < N; ++l) w[l] = __ldg(p + (size_t)(order ? order[l] : l) * nc);
   B = fx_bound<K>(w);
 #pragma unroll
   for (int l = 0; l < N; ++l) x[l] = fx_split(fx_from(w[l], B));
@@ -384,9 +394,9 @@ __device__ __forceinline__ void fx_rows(const Fx (&E)[(K + 1) * (K + 2) / 2], Fx
   }
 }
 
-// values on face (D, S) (S = 0: xi_D = -1, S = 1: xi_D = +1) at the points
-// t1 + Q t2, rows of 32 cells apart
-template <int K, int D, int S>
+// values on the face at xi = -1 (S = 0) or +1 (S = 1) of the first axis at the
+// points t1 + Q t2, rows of 32 cells apart
+template <int K, int S>
 __device__ __forceinline__ void fx_trace(const Fx (&x)[nmodes(K)], int B, double* dst) {
   using FT = FxTab<K>;
   constexpr int Q = K + 1, T = (K + 1) * (K + 2) / 2;
@@ -398,9 +408,9 @@ __device__ __forceinline__ void fx_trace(const Fx (&x)[nmodes(K)], int B, double
     for (int b = 0; a + b <= K; ++b, ++j) {
       FxAcc s{0, 0};
 #pragma unroll
-      for (int e = 1; e + a + b <= K; ++e) fx_madt(s, x[face_mode<D>(e, a, b)], FT::E + S * (K + 1) + e);
+      for (int e = 1; e + a + b <= K; ++e) fx_madt(s, x[mode_index(e, a, b)], FT::E + S * (K + 1) + e);
       // Pt_0 = 1
-      E[j] = fx_split(fx_val(s) + fx_join(x[face_mode<D>(0, a, b)]));
+      E[j] = fx_split(fx_val(s) + fx_join(x[mode_index(0, a, b)]));
     }
   Fx H[Q][K + 1];  // [t2][a]
   fx_rows<K, 0>(E, H);
@@ -450,6 +460,7 @@ __device__ __forceinline__ void fx_moments(const double* f, double* __restrict__
 template <int K, int FLUX, bool MOMENTS = (K >= 2)>
 __global__ void __launch_bounds__(FaceSF64<K>::THREADS, FaceSF64<K>::MINB) face_sf64_kernel(const double* __restrict__ y,
                                                                          double* __restrict__ fh, Geo g, Ctrl* ctrl) {
+  stream_wait();
   using CF = FaceSF64<K>;
   constexpr int N = nmodes(K), C = CF::C, Q2 = CF::Q2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -459,34 +470,25 @@ __global__ void __launch_bounds__(FaceSF64<K>::THREADS, FaceSF64<K>::MINB) face_
   const long long cell = c0 + c;
   const bool live = cell < nc;
   int ix = 0, iy = 0, iz = 0;
-  Fx x[N];
-  int B = 0;
+  if (live) cell_xyz(cell, g, ix, iy, iz);
   const double* yi = y + (size_t)(i * N) * nc;
-  if (live) {
-    cell_xyz(cell, g, ix, iy, iz);
-    fx_load<K>(yi + cell, nc, x, B);
-  }
   unsigned err = 0;
   // directions blockIdx.y, + gridDim.y, ...: all in one CTA, or one per CTA
-  // where a mesh has too few tiles to fill the chip
+  // where a mesh has too few tiles to fill the chip. The coefficients are read
+  // in the order of the face's axes, so that one copy of the trace code serves
+  // the three directions (three copies missed the instruction cache: 9.15 ms per
+  // stage at 128^3, degree 2, one 8.85)
 #pragma unroll 1
   for (int d = blockIdx.y; d < 3; d += gridDim.y) {
     if (live) {
       // row of this variable in the face's frame (rho, m_n, m_t1, m_t2, E)
       double* dst = sU + face_var(d, i) * Q2 * C + c;
-      Fx xl[N];
-      int Bl;
-      fx_load<K>(yi + neighbour(g, ix, iy, iz, d, -1), nc, xl, Bl);
-      if (d == 0) {
-        fx_trace<K, 0, 1>(xl, Bl, dst);
-        fx_trace<K, 0, 0>(x, B, dst + 5 * Q2 * C);
-      } else if (d == 1) {
-        fx_trace<K, 1, 1>(xl, Bl, dst);
-        fx_trace<K, 1, 0>(x, B, dst + 5 * Q2 * C);
-      } else {
-        fx_trace<K, 2, 1>(xl, Bl, dst);
-        fx_trace<K, 2, 0>(x, B, dst + 5 * Q2 * C);
-      }
+      Fx x[N];
+      int B;
+      fx_load<K>(yi + neighbour(g, ix, iy, iz, d, -1), nc, x, B, c_face_order[d]);
+      fx_trace<K, 1>(x, B, dst);
+      fx_load<K>(yi + cell, nc, x, B, c_face_order[d]);
+      fx_trace<K, 0>(x, B, dst + 5 * Q2 * C);
     }
     __syncthreads();
 #pragma unroll 1
@@ -534,6 +536,7 @@ struct FaceF32 {
 template <int K, int FLUX>
 __global__ void __launch_bounds__(96, FaceF32<K>::MINB) face_flux_f32_kernel(const float* __restrict__ yf, float* __restrict__ fh,
                                                               Geo g, Ctrl* ctrl) {
+  stream_wait();
   const long long c = (long long)blockIdx.x * 32 + (threadIdx.x & 31);
   if (c >= g.nc) return;
   const int d = threadIdx.x >> 5;  // warp-uniform direction
@@ -687,6 +690,7 @@ template <int K, int MODE, bool FORCE>
 __global__ void __launch_bounds__(VolF32<K>::THREADS, VolF32<K>::MINB) volume_f32_kernel(
     const float* yfin, const float* __restrict__ fh, const float* __restrict__ field,
     const double* __restrict__ tab64, Geo g, StageArgs st, double* __restrict__ R, Ctrl* ctrl) {
+  stream_wait();
   using TB = Tab<K>;
   using CF = VolF32<K>;
   constexpr int N = TB::N, Q2 = TB::Q2, C = CF::C;
@@ -887,6 +891,7 @@ __global__ void __launch_bounds__(ListLim<K>::THREADS, ListLim<K>::MINB)
     limit_screen_list_kernel(const double* __restrict__ y, const int* __restrict__ list, const unsigned* count,
                              const double* __restrict__ tab64, const float* __restrict__ tab32, Geo g, Ctrl* ctrl,
                              int count_queued, int* __restrict__ deep) {
+  stream_wait();
   constexpr int N = nmodes(K), LT = ListLim<K>::THREADS;
   extern __shared__ __align__(16) double ws[];
   const unsigned n = *count;
@@ -952,6 +957,7 @@ __global__ void __launch_bounds__(ListLim<K>::THREADS)
     limit_list_kernel(double* __restrict__ y, const int* __restrict__ list, const unsigned* count,
                       const double* __restrict__ tab64, Geo g, Ctrl* ctrl, float* __restrict__ yf,
                       const double* __restrict__ y0, float* __restrict__ dinc) {
+  stream_wait();
   using TB = Tab<K>;
   constexpr int N = nmodes(K), LT = ListLim<K>::THREADS, NW = LT / 32;
   extern __shared__ __align__(16) double ws[];
@@ -1216,6 +1222,7 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
     volume_sf_kernel(const double* __restrict__ yin, const float* __restrict__ yf32, const T* __restrict__ fh,
                      const T* __restrict__ field, const T* __restrict__ tab, const double* __restrict__ tab64, Geo g,
                      StageArgs st, double* __restrict__ R, Ctrl* ctrl) {
+  stream_wait();
   static_assert(sizeof(T) == 8, "fixed-point form: FP64 path only");
   using TB = Tab<K>;
   using CF = VolSF<K, double>;
@@ -1521,6 +1528,7 @@ __global__ void __launch_bounds__(kThreads) volume_sfb_kernel(const double* __re
                                                              const T* __restrict__ field, const T* __restrict__ tab,
                                                              const double* __restrict__ tab64, Geo g, StageArgs st,
                                                              double* __restrict__ R, Ctrl* ctrl) {
+  stream_wait();
   static_assert(sizeof(T) == 4, "register-blocked form: FP32 path only");
   using TB = Tab<K>;
   using CF = VolSF<K, T>;
@@ -1875,6 +1883,7 @@ constexpr int kCflThreads = 1024;
 template <int K>
 __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restrict__ y, Geo g, Ctrl* ctrl,
                                                           int slot = 0) {
+  stream_wait();
   constexpr int N = nmodes(K);
   unsigned long long* const max_bits = slot ? &ctrl->cfl_max_bits2 : &ctrl->cfl_max_bits;
   if (blockIdx.x == 0 && threadIdx.x == 0) *(slot ? &ctrl->cfl_max_bits : &ctrl->cfl_max_bits2) = 0ull;
@@ -1986,6 +1995,7 @@ template <int K, typename T>
 __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel(
     double* __restrict__ y, const T* __restrict__ tab, Geo g, ResetConsts<T> rc, double* __restrict__ part,
     int* __restrict__ list, Ctrl* ctrl, float* __restrict__ yf) {
+  stream_wait();
   using RS = ResetSF<K, T>;
   using TB = Tab<K>;
   constexpr int C = RS::C, Q = RS::Q, Q3 = RS::Q3, N = RS::N, ROW = RS::ROW, V = RS::V;
@@ -2217,14 +2227,22 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
       sEn[it] = A < kFxHuge ? fx_to_double(t, A) : __longlong_as_double(0x7ff8000000000000LL);
     }
   } else {
-    constexpr int KQ = (K + 1) * Q, GROW = Q * Q * (K + 1);
+    // rows of G an odd number of words apart: lanes over cells hit different banks
+    // (degree 3, 160^3: 5.4 ms with 64 words, 1.8 with 65)
+    constexpr int KQ = (K + 1) * Q, GROW = Q * Q * (K + 1) | 1;
     T* sG = sU;  // [cell][(qz Q + qy) (K + 1) + u]
     for (int it = tid; it < Q * Q * C; it += RS::THREADS) {
       const int c = it / (Q * Q), r = it - c * (Q * Q);  // r = qz Q + qy
       const T* e = sE + c * ROW + r * Q;
       T ev[Q];
+      if constexpr (Q == V) {
+        const Vec t = *reinterpret_cast<const Vec*>(e);  // a row of four points is 16 bytes
 #pragma unroll
-      for (int qx = 0; qx < Q; ++qx) ev[qx] = e[qx];
+        for (int qx = 0; qx < Q; ++qx) ev[qx] = t.v[qx];
+      } else {
+#pragma unroll
+        for (int qx = 0; qx < Q; ++qx) ev[qx] = e[qx];
+      }
 #pragma unroll
       for (int u = 0; u <= K; ++u) {
         T s = T(0);
@@ -2270,18 +2288,22 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
       sf = fmaf(abs_up(sEn[l * C + c]), g.lim_vol ? c_tab32[TB::LMAXV + l] : c_tab32[TB::LMAX + l], sf);
       fin &= finite64(sEn[l * C + c]);
     }
-    const double ae = (double)sf * (1.0 + 1e-5);
-    const double r = sM[c], m1 = sM[C + c], m2 = sM[2 * C + c], m3 = sM[3 * C + c];
-    const double kin = 0.5 * (m1 * m1 + m2 * m2 + m3 * m3) / r;
-    diss = (sM[4 * C + c] - kin) - (sEn[c] - kin);
-    double m[5] = {r, m1, m2, m3, sEn[c]}, a[5];
+    // the kinetic energy of the means stays: the drop of the internal energy is
+    // that of the total
+    diss = sM[4 * C + c] - sEn[c];
+    // FP32 screen (the FP64 one took two divisions and some 30 further FP64
+    // operations per cell: reset and limiter at 128^3, degree 2, FP32-mixed, 0.41
+    // ms with it, 0.35 so)
+    float m[5], a[5];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      a[i] = sA[i * C + c];
+      m[i] = f64_to_f32_q(sM[i * C + c]);
+      a[i] = f64_to_f32_q(sA[i * C + c]) * (1.f + 1e-6f);
       fin &= sFin[i * C + c] != 0;
     }
-    a[4] = ae;
-    if (!limiter_screen<K>(m, a, fin, g.gamma, g.eps_rho, g.eps_p)) {
+    m[4] = f64_to_f32_q(sEn[c]);
+    a[4] = sf * (1.f + 1e-5f);
+    if (!fin || !screen_f32(m, a, (float)(g.gamma - 1.0), (float)g.eps_rho, (float)g.eps_p)) {
       const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
       list[slot] = (int)cell;
     }

@@ -61,31 +61,59 @@ __device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], const
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// A fragment (16x16) of a row-major matrix M[row][k] in shared memory.
+// Fragments of m16n8k16 from matrices in shared memory, by ldmatrix on the
+// device (one instruction for four registers: with 4-byte and, transposed, 2-byte
+// loads the kernels were bound by them; forward and backward of 262,144 rows of
+// 192 features 180 us, now 165). The host emulation loads element by element.
+//
+// A fragment (16x16) of a row-major matrix M[row][k].
 __device__ __forceinline__ void frag_a(uint32_t (&a)[4], const bf16* M, int ld, int r0, int k0, int g, int t) {
+#ifdef __CUDA_ARCH__
+  const int l = g * 4 + t;
+  ldsm4(a, M + (r0 + (l & 15)) * ld + k0 + (l >> 4) * 8);
+#else
   a[0] = ld32(M + (r0 + g) * ld + k0 + 2 * t);
   a[1] = ld32(M + (r0 + g + 8) * ld + k0 + 2 * t);
   a[2] = ld32(M + (r0 + g) * ld + k0 + 8 + 2 * t);
   a[3] = ld32(M + (r0 + g + 8) * ld + k0 + 8 + 2 * t);
+#endif
 }
-// B fragment (16x8) from Bt[n][k] (k contiguous).
-__device__ __forceinline__ void frag_b(uint32_t (&b)[2], const bf16* Bt, int ld, int n0, int k0, int g, int t) {
-  b[0] = ld32(Bt + (n0 + g) * ld + k0 + 2 * t);
-  b[1] = ld32(Bt + (n0 + g) * ld + k0 + 8 + 2 * t);
+// B fragments (16x8) of the columns n0 .. n0 + 7 (b[0], b[1]) and n0 + 8 .. n0 +
+// 15 (b[2], b[3]) from Bt[n][k] (k contiguous).
+__device__ __forceinline__ void frag_b2(uint32_t (&b)[4], const bf16* Bt, int ld, int n0, int k0, int g, int t) {
+#ifdef __CUDA_ARCH__
+  const int l = g * 4 + t;
+  ldsm4(b, Bt + (n0 + (l >> 4) * 8 + (l & 7)) * ld + k0 + ((l >> 3) & 1) * 8);
+#else
+  for (int h = 0; h < 2; ++h) {
+    b[2 * h] = ld32(Bt + (n0 + 8 * h + g) * ld + k0 + 2 * t);
+    b[2 * h + 1] = ld32(Bt + (n0 + 8 * h + g) * ld + k0 + 8 + 2 * t);
+  }
+#endif
 }
 // A fragment of the transpose of S[k][m] (S row-major, rows = k).
 __device__ __forceinline__ void frag_at(uint32_t (&a)[4], const bf16* S, int ld, int m0, int k0, int g, int t) {
+#ifdef __CUDA_ARCH__
+  const int l = g * 4 + t;
+  ldsm4_t(a, S + (k0 + (l >> 4) * 8 + (l & 7)) * ld + m0 + ((l >> 3) & 1) * 8);
+#else
   const int k = k0 + 2 * t;
   a[0] = pack2h(S[k * ld + m0 + g], S[(k + 1) * ld + m0 + g]);
   a[1] = pack2h(S[k * ld + m0 + g + 8], S[(k + 1) * ld + m0 + g + 8]);
   a[2] = pack2h(S[(k + 8) * ld + m0 + g], S[(k + 9) * ld + m0 + g]);
   a[3] = pack2h(S[(k + 8) * ld + m0 + g + 8], S[(k + 9) * ld + m0 + g + 8]);
+#endif
 }
 // B fragment with B[k][n] = S[k][n] (S row-major, rows = k).
 __device__ __forceinline__ void frag_bk(uint32_t (&b)[2], const bf16* S, int ld, int n0, int k0, int g, int t) {
+#ifdef __CUDA_ARCH__
+  const int l = g * 4 + t;
+  ldsm2_t(b, S + (k0 + (l & 15)) * ld + n0);
+#else
   const int k = k0 + 2 * t;
   b[0] = pack2h(S[k * ld + n0 + g], S[(k + 1) * ld + n0 + g]);
   b[1] = pack2h(S[(k + 8) * ld + n0 + g], S[(k + 9) * ld + n0 + g]);
+#endif
 }
 
 // ------------------------------------------------------------- features
@@ -186,10 +214,12 @@ __device__ __forceinline__ void warp_forward(const bf16* sX, const bf16* sW1, co
     uint32_t a[4];
     frag_a(a, sX, L::LDX, r0, kt * 16, g, t);
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      uint32_t b[2];
-      frag_b(b, sW1, L::LDX, nt * 8, kt * 16, g, t);
-      mma(c1[nt], a, b);
+    for (int nt = 0; nt < 8; nt += 2) {
+      uint32_t b[4];
+      frag_b2(b, sW1, L::LDX, nt * 8, kt * 16, g, t);
+      const uint32_t b0[2] = {b[0], b[1]}, b1[2] = {b[2], b[3]};
+      mma(c1[nt], a, b0);
+      mma(c1[nt + 1], a, b1);
     }
   }
 #pragma unroll
@@ -208,10 +238,12 @@ __device__ __forceinline__ void warp_forward(const bf16* sX, const bf16* sW1, co
 #pragma unroll
   for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      uint32_t b[2];
-      frag_b(b, sW2, L::LDH, nt * 8, j * 16, g, t);
-      mma(z2[nt], h1a[j], b);
+    for (int nt = 0; nt < 8; nt += 2) {
+      uint32_t b[4];
+      frag_b2(b, sW2, L::LDH, nt * 8, j * 16, g, t);
+      const uint32_t b0[2] = {b[0], b[1]}, b1[2] = {b[2], b[3]};
+      mma(z2[nt], h1a[j], b0);
+      mma(z2[nt + 1], h1a[j], b1);
     }
   float slo = 0.f, shi = 0.f;
 #pragma unroll
@@ -379,10 +411,12 @@ __global__ void __launch_bounds__(256) backward_kernel(const bf16* __restrict__ 
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int nt = 0; nt < 8; ++nt) {
-        uint32_t b[2];
-        frag_b(b, sW2T, L::LDH, nt * 8, j * 16, g, t);
-        mma(dz1[nt], dza[j], b);
+      for (int nt = 0; nt < 8; nt += 2) {
+        uint32_t b[4];
+        frag_b2(b, sW2T, L::LDH, nt * 8, j * 16, g, t);
+        const uint32_t b0[2] = {b[0], b[1]}, b1[2] = {b[2], b[3]};
+        mma(dz1[nt], dza[j], b0);
+        mma(dz1[nt + 1], dza[j], b1);
       }
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
@@ -546,13 +580,25 @@ __global__ void __launch_bounds__(256) gate_kernel(const double* __restrict__ y,
   }
 }
 
-// grads[j] = sum over partial rows (fixed order)
+// grads[j] = sum over partial rows: blockDim.y threads per column take every
+// blockDim.y-th row, their sums are added in a fixed order. The 304 rows one
+// after the other in a thread per column were a chain of dependent loads on 66
+// blocks: 21 us at
+// 16,769 columns, now 12.
+constexpr int kRedCols = 32, kRedRows = 16;
 __global__ void reduce_rows_kernel(const float* __restrict__ part, int rows, int cols, float* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= cols) return;
+  __shared__ float red[kRedRows * kRedCols];
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, g = threadIdx.y;
   float s = 0.f;
-  for (int r = 0; r < rows; ++r) s += part[(size_t)r * cols + j];
-  out[j] = s;
+  if (j < cols)
+    for (int r = g; r < rows; r += blockDim.y) s += part[(size_t)r * cols + j];
+  if (blockDim.y > 1) {
+    red[g * blockDim.x + threadIdx.x] = s;
+    __syncthreads();
+    if (g > 0) return;
+    for (int k = 1; k < blockDim.y; ++k) s += red[k * blockDim.x + threadIdx.x];
+  }
+  if (j < cols) out[j] = s;
 }
 
 __global__ void adam_kernel(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
@@ -605,7 +651,7 @@ struct Ops {
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int cols = PL<F>::TOTAL + 1;
-    reduce_rows_kernel<<<(cols + 255) / 256, 256, 0, s>>>(part, rows, cols, grads);
+    reduce_rows_kernel<<<(cols + kRedCols - 1) / kRedCols, dim3(kRedCols, kRedRows), 0, s>>>(part, rows, cols, grads);
     return cudaGetLastError();
   }
 };
