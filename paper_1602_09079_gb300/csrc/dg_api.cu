@@ -1309,6 +1309,9 @@ int noalloc_setup(int dev, int k, void** scratch) {
     }
     for (int i = 0; i < TAB_STRIDE; ++i) g_noalloc_tab32[i] = (float)g_noalloc_tab64[i];
     if (launchers_for(k).upload(g_noalloc_tab64, g_noalloc_tab32) != cudaSuccess) return DG_ERR_CUDA;
+    // the bit below speaks for the fused kernels' tables too
+    const FusedLaunchers F = fused_for(k);
+    if (F.upload && F.upload(g_noalloc_tab64) != cudaSuccess) return DG_ERR_CUDA;
     g_uploaded[k] |= 1ull << dev;
   }
   return DG_OK;

@@ -3,6 +3,10 @@ cell, one row or one plane, tiles cut at both sides, segments of one and two
 planes and a last segment that is shorter; orders 2 to 4, both fluxes, with
 and without driving, the limiter at rest. Against the oracle with the FP32-mixed
 path's bars: R 2e-5, a step's state 1e-6."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -10,6 +14,7 @@ import oracle
 import synthetic as syn
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 G = syn.GAMMA
 HIGH = {2: 0.02, 3: 0.012, 4: 0.006}  # density and pressure stay positive at every point
 
@@ -45,3 +50,35 @@ def test_step_and_rhs(order, n, flux, force):
     s.step(dt)
     s.check()
     assert normwise(s.get_state(), w1) <= 1e-6
+
+
+@pytest.mark.parametrize("order", [2, 3, 4])
+def test_step_after_noalloc_call_came_first(order):
+    """In a new process the first call of an order is dg_rhs_noalloc, which
+    uploads the order's tables; the mixed step that follows finds the fused
+    kernels' tables as well. Against the FP64 step, whose own bar is 1e-12."""
+    code = f"""
+import sys
+sys.path[:0] = [{ROOT!r}, {ROOT!r} + "/tests"]
+import numpy as np, torch, synthetic as syn, paper_1602_09079_gb300 as dg
+n, order = (9, 7, 5), {order}
+N = order * (order + 1) * (order + 2) // 6
+y = torch.ones(5 * N * 315, dtype=torch.float64, device="cuda")
+R = torch.empty_like(y)
+dg.dg_rhs_noalloc(n, order, syn.GAMMA, dg.DG_PREC_MIXED, y, R, 0)
+torch.cuda.synchronize()
+w = syn.random_state(n, N, syn.GAMMA, seed=order, high={HIGH[order]})
+out = []
+for prec in (dg.DG_PREC_FP64, dg.DG_PREC_MIXED):
+    s = dg.Solver(n, order, syn.GAMMA)
+    s.set_precision(prec)
+    s.set_state(w)
+    s.step(1e-3)
+    s.check()
+    out.append(s.get_state())
+for i in range(5):
+    a, b = out[1][..., i, :], out[0][..., i, :]
+    assert np.max(np.abs(a - b)) <= 1e-6 * np.max(np.abs(b)), i
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
