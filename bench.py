@@ -218,24 +218,25 @@ def roofline_entry(kind, achieved, peak, unit, bound, traffic=None):
             "frac": (achieved / peak) if peak else None, "traffic": traffic}
 
 
-def step_roofline(k, mixed, nc, ms_per_step, hbm_gbs):
+def step_roofline(k, mixed, nc, ms_per_step, hbm_gbs, fp64_peak=None):
     """Whole-step roofline: the algorithmic work of the step's three RK
     stages (roofline.step_min_bytes: read y_s, y_0, write y_{s+1} in FP64;
     3 x roofline.stage_flops, sum-factorised) plus the energy reset (read the
     density and momentum modes and the energy mean, write the energy modes)
     and the CFL reduction (five means), over the measured step time; bound
-    by the larger of the ALU time (FP32 peak on the mixed path, FP64 on the
-    plain one) and the HBM time."""
+    by the larger of the ALU time (FP32 peak on the mixed path; on the plain
+    one fp64_peak, the FP64 pipe's rate if None) and the HBM time."""
     from paper_1602_09079_gb300 import roofline as rl
     N = (k + 1) * (k + 2) * (k + 3) // 6
     sec = ms_per_step * 1e-3
     byts = (rl.step_min_bytes(k) + (4 * N + 1 + N) * 8 + 5 * 8) * nc
     flops = 3 * rl.stage_flops(k, True) * nc
-    peak = rl.FP32_PEAK if mixed else rl.FP64_PEAK
+    peak = rl.FP32_PEAK if mixed else fp64_peak or rl.FP64_PEAK
     t_alu = flops / peak
     t_hbm = byts / (hbm_gbs * 1e9) if hbm_gbs else None
     out = {"bytes_per_step": byts, "flops_per_step": flops, "achieved_gbs": byts / sec / 1e9,
-           "achieved_tflops": flops / sec / 1e12, "peak_source": rl.PEAK_SOURCE,
+           "achieved_tflops": flops / sec / 1e12,
+           "peak_source": rl.FP64_FIXED_SOURCE if fp64_peak and not mixed else rl.PEAK_SOURCE,
            "impl_bytes_per_step": rl.step_bytes(k, mixed) * nc}
     if t_hbm is None:
         out.update({"bound": None, "achieved": None, "peak": None, "unit": None, "frac": None})
@@ -394,16 +395,17 @@ def run_ours(args):
         nvol, msvol = kst["volume"]
         nface, msface = kst["face_flux"]
         stage_ms = (msvol + msface) / nvol
-        peak = rl.FP32_PEAK if tsize == 4 else rl.FP64_PEAK
+        fixed = tsize == 8 and k >= 1  # order 1 has no contraction: plain FP64
+        peak = rl.FP32_PEAK if tsize == 4 else rl.FP64_FIXED_PEAK if fixed else rl.FP64_PEAK
         e = rl.stage_roofline(k, True, nc, stage_ms, hbm, peak)
-        e["peak_source"] = rl.PEAK_SOURCE
+        e["peak_source"] = rl.FP64_FIXED_SOURCE if fixed else rl.PEAK_SOURCE
         fused = tsize == 4 and nface == 0
         if fused:
             kname = f"fused_f32_kernel<{k}, true, {1 if args.flux == 'exact' else 0}>"
             e["kernel"] = kname + " (stage, forcing; face fluxes, volume integral and stage update in one launch)"
             e["impl_bytes_per_launch"] = rl.fused_impl_bytes(k, True) * nc
         else:
-            sumfact = k >= 2
+            sumfact = k >= (1 if tsize == 8 else 2)
             kname = (f"volume_f32_kernel<{k}, 1, 1>" if (tsize == 4 and k <= 2)
                      else f"volume_{('sfb_' if tsize == 4 else 'sf_') if sumfact else ''}kernel<{k}, "
                      f"{'double' if tsize == 8 else 'float'}, 1, 1>")
@@ -458,7 +460,8 @@ def run_ours(args):
                 "ms_per_step": r_64["ms_max"] / args.steps,
                 "dtype": "f64",
                 "roofline": kernel_roofline("fp64", 8) if "fp64" in results else None,
-                "step_roofline": (step_roofline(k, False, nc, r_64["ms_max"] / args.steps, hbm)
+                "step_roofline": (step_roofline(k, False, nc, r_64["ms_max"] / args.steps, hbm,
+                                                rl.FP64_FIXED_PEAK if k else None)
                                   if "fp64" in results else None),
                 "clocks": r_64["clocks"],
                 "gpu_launches": sum(v[0] for v in r_64["launches"].values()),

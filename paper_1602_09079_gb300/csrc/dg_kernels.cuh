@@ -1875,10 +1875,12 @@ __global__ void __launch_bounds__(kThreads) limit_kernel(double* __restrict__ y,
 // FP64 s (a few roundings, the pressure's amplified at most 199x by the
 // cancellation, halved by the square root), so the cell holding the
 // block's FP64 maximum is always among the re-evaluated ones. Blocks combine
-// by one atomicMax on the bit pattern of the non-negative double. Blocks of
-// 1024 cells: a block's re-evaluations (usually the one cell that holds its
-// maximum) occupy the FP64 pipe for a whole warp, so fewer, larger blocks.
-constexpr int kCflThreads = 1024;
+// by one atomicMax on the bit pattern of the non-negative double; inside a
+// block the maxima are compared as bit patterns too, because a warp's FP64
+// comparison holds the FP64 pipe for 16 clocks. 128^3: 39 us, from 60 us with
+// FP64 comparisons and blocks of 1024 (bit patterns and 1024: 42; the means at
+// the HBM rate: 12); degree 3, 160^3: 67 us from 106 (512 threads: 70).
+constexpr int kCflThreads = 256;
 
 template <int K>
 __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restrict__ y, Geo g, Ctrl* ctrl,
@@ -1909,7 +1911,7 @@ __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restri
     trusted = rf >= 1e-30f && rf <= 1e30f && Ef <= 1e30f && kin <= 0.99f * Ef && prf >= 1e-30f && sf <= 3e38f;
   }
   __shared__ float s_wf[kCflThreads / 32];
-  __shared__ double s_w[kCflThreads / 32];
+  __shared__ unsigned long long s_w[kCflThreads / 32];
   __shared__ unsigned s_err;
   float mf = trusted ? sf : 0.f;
 #pragma unroll
@@ -1920,7 +1922,9 @@ __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restri
   mf = s_wf[0];
 #pragma unroll
   for (int w = 1; w < kCflThreads / 32; ++w) mf = fmaxf(mf, s_wf[w]);
-  double smax = 0.0;
+  // the FP64 maxima as bit patterns (non-negative doubles order like integers): the
+  // FP64 pipe takes 16 clocks for a warp's comparison
+  unsigned long long smax = 0ull;
   unsigned e = 0;
   if (c < nc && (!trusted || sf >= mf * (1.f - 1e-3f))) {
     const double ir = 1.0 / r;
@@ -1929,21 +1933,28 @@ __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restri
       e = (isfinite(r) && isfinite(pr)) ? ERRB_POSITIVITY : ERRB_NONFINITE;
     } else {
       const double cs = sqrt(g.gamma * pr * ir);
-      smax = (fabs(m1) * ir + cs) * g.inv_dx[0] + (fabs(m2) * ir + cs) * g.inv_dx[1] +
-             (fabs(m3) * ir + cs) * g.inv_dx[2];
+      const double sd = (fabs(m1) * ir + cs) * g.inv_dx[0] + (fabs(m2) * ir + cs) * g.inv_dx[1] +
+                        (fabs(m3) * ir + cs) * g.inv_dx[2];
+      if (sd > 0.0) smax = (unsigned long long)__double_as_longlong(sd);
     }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, smax, o);
+    if (v > smax) smax = v;
+  }
   if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = smax;
   if (e) atomicOr(&s_err, e);
   __syncthreads();
   if (threadIdx.x < 32) {
-    double v = threadIdx.x < kCflThreads / 32 ? s_w[threadIdx.x] : 0.0;
+    unsigned long long v = threadIdx.x < kCflThreads / 32 ? s_w[threadIdx.x] : 0ull;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+      if (u > v) v = u;
+    }
     if (threadIdx.x == 0) {
-      atomicMax(max_bits, (unsigned long long)__double_as_longlong(v));
+      atomicMax(max_bits, v);
       if (s_err) atomicOr(&ctrl->err, s_err);
     }
   }
@@ -2366,10 +2377,11 @@ __global__ void __launch_bounds__(kThreads) project_kernel(const double* __restr
 // field) as sum_l m_l a_l with the driving field's projection a_l = sum_q a
 // phi_l omega_q / 8, sum-factorised in fixed point: the field is read once and
 // 3 N FP64 multiply-adds remain of 3 Q^3 (N + 1). 64^3, degree 2, FP32 field:
-// 125 us, the dense FP64 sums took 470.
+// 107 us, the dense FP64 sums took 470. Registers for 3 CTAs per SM (2: 125
+// us; 4: 107).
 // part[j * gridDim.x + b], j = 0, 1, 2.
 template <int K, typename T>
-__global__ void __launch_bounds__(256) diag_partial_kernel(const double* __restrict__ y, const T* __restrict__ field,
+__global__ void __launch_bounds__(256, 3) diag_partial_kernel(const double* __restrict__ y, const T* __restrict__ field,
                                                            const double* __restrict__ tab64, Geo g, int force,
                                                            double* __restrict__ part) {
   using TB = Tab<K>;

@@ -7,9 +7,8 @@ namespace dg {
 
 // Launch with programmatic stream serialisation: the chip sets the kernel up
 // while its predecessor drains, which hides most of a launch on small meshes
-// (8^3, FP64,
-// order 2, 13 kernels per step: 105 us with plain launches, 74 so). The kernel's first
-// statement is stream_wait().
+// (8^3, FP64, order 2, 13 kernels per step: 105 us with plain launches, 74 so).
+// The kernel's first statement is stream_wait().
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t c{};
