@@ -412,6 +412,9 @@ def run_ours(args):
             e["kernel"] = kname + " (stage, forcing) + its face kernel"
             e["impl_bytes_per_launch"] = (rl.volume_bytes(k, tsize, True, shadow=tsize == 4)
                                           + rl.face_bytes(k, tsize)) * nc
+            if fixed:  # the face buffer holds moments: T values per variable and direction in place of Q^2
+                T = (k + 1) * (k + 2) // 2
+                e["impl_bytes_per_launch"] -= 2 * 15 * ((k + 1) ** 2 - T) * 8 * nc
         # the captured FP64 traffic is that of the HLLC face kernel: no entry
         # for the exact-flux path
         tr = None if (args.flux == "exact" and not fused) else ncu_traffic().get(kname)
