@@ -386,7 +386,7 @@ def run_ours(args):
 
     def kernel_roofline(prec_name, tsize):
         """Roofline of one RK stage: the stage kernels' time per stage (the
-        fused kernel on the mixed path at degrees 2-3; face and volume kernels
+        fused kernel on the mixed path at degrees 1-3; face and volume kernels
         otherwise) against the method's algorithmic bytes (read y_s and y_0,
         write y_{s+1} in FP64) and sum-factorised flops of a stage
         (roofline.stage_roofline); traffic = the ncu DRAM bytes of the timed
