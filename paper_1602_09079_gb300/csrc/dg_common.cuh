@@ -416,12 +416,18 @@ __device__ __forceinline__ int face_var(int d, int i) {
 // h cl + l ch into mid; l cl stays below one unit), a sum one shift at its
 // end. Partial sums may wrap, sums may not: the bounds stand at each caller.
 struct Fx {
-  int h, l;  // value h 2^30 + l, 0 <= l < 2^30
+  int h, l;  // value h 2^30 + l, 0 <= l < 2^30 (fx_split_signed: |l| <= 2^29)
 };
 struct FxAcc {
   long long hi, mid;  // value (hi 2^60 + mid 2^30) 2^-58
 };
 __device__ __forceinline__ Fx fx_split(long long r) { return {(int)(r >> 30), (int)(r & 0x3fffffff)}; }
+// the same with -2^29 <= l < 2^29, for |r| < 2^60.9: where many products go into
+// one sum, low limbs that are never negative would not cancel in its mid
+__device__ __forceinline__ Fx fx_split_signed(long long r) {
+  const int l = ((int)(r & 0x3fffffff) ^ 0x20000000) - 0x20000000;
+  return {(int)((r - l) >> 30), l};
+}
 __device__ __forceinline__ long long fx_join(Fx x) { return (long long)x.h * (1 << 30) + x.l; }
 __device__ __forceinline__ void fx_mad(FxAcc& a, Fx x, int ch, int cl) {
   a.hi += (long long)x.h * ch;

@@ -933,14 +933,19 @@ __global__ void __launch_bounds__(ListLim<K>::THREADS, ListLim<K>::MINB)
 
 // coefficients of variable i of a cell, w[5 N] in shared memory, in fixed point
 // to x (lanes: modes); returns the exponent. sum_l |phi_l| over the cell stays
-// below 2^3, 2^5 and 2^6 at degrees 1 to 3.
+// below 2^3, 2^5 and 2^6 at degrees 1 to 3, so that |x| < 2^55 at degree 3 and a
+// point value stays below 2^61. The N - 1 products of a point value go into one
+// FxAcc: with signed limbs on both sides |mid| <= sum_l |x.l ch| + |x.h cl| <=
+// 2^29 2^28 sum_l |phi_l| + (N - 1) 2^25 2^29 <= 40.7 2^57 + 19 2^54 < 2^62.5.
+// (Low limbs that are never negative reached 40.7 2^58 > 2^63 where all phi_l
+// are positive.)
 template <int K>
 __device__ __forceinline__ int fx_cell(const double* w, Fx* x, int lane) {
   constexpr int N = nmodes(K);
   unsigned mx = 0;
   for (int l = 0; l < N; ++l) mx = max(mx, (unsigned)__double2hiint(w[l]) & 0x7fffffffu);
   const int B = max(kFxTiny, bexp(mx) + (K == 1 ? 3 : K == 2 ? 5 : 6));
-  if (lane < N) x[lane] = fx_split(fx_from(w[lane], B));
+  if (lane < N) x[lane] = fx_split_signed(fx_from(w[lane], B));
   return B;
 }
 
@@ -993,7 +998,7 @@ __global__ void __launch_bounds__(ListLim<K>::THREADS)
       FxAcc a{0, 0};
 #pragma unroll
       for (int l = 1; l < N; ++l) {
-        const Fx p = fx_split(fx_from(__ldg(ph + l), 1025));  // units of 2^-58
+        const Fx p = fx_split_signed(fx_from(__ldg(ph + l), 1025));  // units of 2^-58
         fx_mad(a, x[l], p.h, p.l);
       }
       const double r = fx_to_double(fx_val(a) + fx_join(x[0]), B[0]);
@@ -1025,7 +1030,7 @@ __global__ void __launch_bounds__(ListLim<K>::THREADS)
       for (int i = 0; i < 5; ++i) a[i] = {0, 0};
 #pragma unroll
       for (int l = 1; l < N; ++l) {
-        const Fx p = fx_split(fx_from(__ldg(ph + l), 1025));
+        const Fx p = fx_split_signed(fx_from(__ldg(ph + l), 1025));
 #pragma unroll
         for (int i = 0; i < 5; ++i) fx_mad(a[i], x[i * N + l], p.h, p.l);
       }
