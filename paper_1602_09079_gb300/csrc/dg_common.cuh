@@ -369,27 +369,45 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
   return 1.f / std::sqrt(x);
 #endif
 }
+// Pressure part of the limiter's FP32 screens: true when gm1 (E - |m|^2 / (2
+// rho)) clears ep for every rho >= rlo > 0, E >= elo and |m_j| <= mh_j,
+// multiplied through by the density bound, with a 1e-5 margin relative to eabs >=
+// |E|, which covers the FP32 rounding of the inputs and of the test. The products
+// rho E and m^2 leave the range of binary32 in units as common as g / cm^3 (and 0
+// >= 0 would hold), so the test runs on rho, E and m scaled by powers of two 2^a,
+// 2^b and 2^((a + b) / 2) that bring rlo and eabs near 1: where the plain products
+// are in range the outcome is the same, bit for bit. Bounds below 2^-103 or
+// above 2^125, zeros, infinities and NaNs fail: the caller's next, FP64 test decides.
+__device__ __forceinline__ bool pressure_clear_f32(float rlo, float elo, float eabs, const float (&mh)[3], float gm1,
+                                                   float ep) {
+  // biased exponents (a set sign makes them large), their sum made even
+  const int xr = (int)(__float_as_uint(rlo) >> 23), x4 = (int)(__float_as_uint(eabs) >> 23);
+  if ((unsigned)(xr - 24) > 228u || (unsigned)(x4 - 24) > 228u) return false;
+  const int xe = x4 + ((xr + x4) & 1);
+  const float sr = __uint_as_float((unsigned)(254 - xr) << 23), se = __uint_as_float((unsigned)(254 - xe) << 23);
+  const float sm = __uint_as_float((unsigned)(254 - (xr + xe) / 2) << 23);
+  float k2 = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) k2 = fmaf(mh[a] * sm, mh[a] * sm, k2);
+  k2 *= 0.5f;
+  const float r = rlo * sr;
+  const float lhs = gm1 * fmaf(elo * se, r, -k2);
+  const float rhs = fmaf(ep * se, r, 1e-5f * gm1 * fmaf(eabs * se, r, k2));
+  return lhs >= rhs;
+}
+
 // Sufficient limiter screen in FP32 from the cell means m and the excursion
 // bounds s_i >= sum_{l>=1} |w_il| max|phi_l|: true when the density and the
 // pressure provably stay above the floors at every point of the limiter's
-// point set (same bounds as the FP64 screen, multiplied through by the
-// density bound, with a 1e-5 relative margin that covers the FP32 rounding
-// of the inputs and of the test). NaN inputs fail.
+// point set (same bounds as the FP64 screen, with a 1e-5 relative margin that
+// covers the FP32 rounding of the inputs and of the test). NaN inputs fail, and
+// so do states outside the range of pressure_clear_f32.
 __device__ __forceinline__ bool screen_f32(const float* m, const float* s, float gm1, float er, float ep) {
   const float r = m[0];
   const float rlo = r - s[0];
   if (!(rlo >= er + 1e-5f * (fabsf(r) + s[0]))) return false;
-  float k2 = 0.f;
-#pragma unroll
-  for (int a = 1; a <= 3; ++a) {
-    const float mh = fabsf(m[a]) + s[a];
-    k2 = fmaf(mh, mh, k2);
-  }
-  k2 *= 0.5f;
-  const float elo = m[4] - s[4];
-  const float lhs = gm1 * fmaf(elo, rlo, -k2);
-  const float rhs = fmaf(ep, rlo, 1e-5f * gm1 * fmaf(fabsf(m[4]) + s[4], rlo, k2));
-  return lhs >= rhs;
+  const float mh[3] = {fabsf(m[1]) + s[1], fabsf(m[2]) + s[2], fabsf(m[3]) + s[3]};
+  return pressure_clear_f32(rlo, m[4] - s[4], fabsf(m[4]) + s[4], mh, gm1, ep);
 }
 
 // position of conserved variable i in the frame of a face normal to axis d:
@@ -978,6 +996,33 @@ __device__ __forceinline__ double positivity_tau(const double* qb, const double*
   return tau;
 }
 
+// x 2^de by its exponent field: exact; zeros, subnormals and results below 2^-1022
+// give a signed zero, results above the range a number of at least 2^1023
+__device__ __forceinline__ double exp_add(double x, int de) {
+  const int hi = __double2hiint(x), b = bexp((unsigned)hi), n = min(b + de, 2046);
+  const bool zero = b == 0 || n <= 0;
+  return __hiloint2double((int)((unsigned)hi & 0x80000000u) | (zero ? 0 : (hi & 0xfffff) | (n << 20)),
+                          zero ? 0 : __double2loint(x));
+}
+
+// A cell's own units for the FP32 point screens, from its mean density and energy:
+// powers of two 2^r, 2^e and 2^((r + e) / 2) that bring rho, E and the momenta near
+// 1. rho E and m^2 scale alike, so the screens decide as they would in binary32
+// of unlimited range. Means near the ends of the FP64 range (ok unset) are left
+// to the FP64 limiter.
+struct LimUnits {
+  int r, m, e;
+  bool ok;
+  __device__ __forceinline__ LimUnits(double rho, double E) {
+    const int br = bexp((unsigned)__double2hiint(rho)), be = bexp((unsigned)__double2hiint(E));
+    ok = (unsigned)(br - 64) <= 1900u && (unsigned)(be - 64) <= 1900u;
+    r = 1023 - br;
+    e = 1023 - be - ((br + be) & 1);
+    m = (r + e) / 2;
+  }
+  __device__ __forceinline__ int of(int i) const { return i == 0 ? r : (i == 4 ? e : m); }
+};
+
 // Second sufficient test of the positivity limiter, for cells whose modal
 // bound fails: density and pressure at every point of the limiter's point
 // set (S, and the volume Gauss points when vol), evaluated in FP32 from the
@@ -989,7 +1034,8 @@ __device__ __forceinline__ double positivity_tau(const double* qb, const double*
 // the density and the pressure (bounded below through the density's lower
 // and the momenta's upper bounds, multiplied through by the density bound)
 // must clear the floors with a further 1e-5 relative margin, which covers
-// the FP32 rounding of the test itself. True when the cell provably needs
+// the FP32 rounding of the test itself. The test runs in the cell's own units
+// (LimUnits), so that no product of the values leaves the range of binary32. True when the cell provably needs
 // no limiting (theta1 = theta2 = 1): the FP64 limiter would leave it as it is.
 template <int K>
 __device__ bool point_screen_f32(const double* w, long long stride, const float* __restrict__ tab32,
@@ -997,14 +1043,16 @@ __device__ bool point_screen_f32(const double* w, long long stride, const float*
                                  int vol) {
   using TB = Tab<K>;
   constexpr int N = TB::N;
+  const LimUnits un(mean[0], mean[4]);
+  if (!un.ok) return false;
   float wf[5 * N];
 #pragma unroll
-  for (int j = 0; j < 5 * N; ++j) wf[j] = f64_to_f32(w[j * stride]);
+  for (int j = 0; j < 5 * N; ++j) wf[j] = f64_to_f32(exp_add(w[j * stride], un.of(j / N)));
   float e[5];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) e[i] = f64_to_f32(2e-6 * (fabs(mean[i]) + sabs[i]));
-  const float thr_r = f64_to_f32(eps_r * (1.0 + 1e-6) + 1e-5 * (fabs(mean[0]) + sabs[0]));
-  const float eps_pf = f64_to_f32(eps_p * (1.0 + 1e-6));
+  for (int i = 0; i < 5; ++i) e[i] = f64_to_f32(exp_add(2e-6 * (fabs(mean[i]) + sabs[i]), un.of(i)));
+  const float thr_r = f64_to_f32(exp_add(eps_r * (1.0 + 1e-6) + 1e-5 * (fabs(mean[0]) + sabs[0]), un.r));
+  const float eps_pf = f64_to_f32(exp_add(eps_p * (1.0 + 1e-6), un.e));
   const float gm1 = f64_to_f32(gamma - 1.0);
   const int npts = TB::NL + (vol ? TB::Q3 : 0);
   for (int s = 0; s < npts; ++s) {

@@ -829,18 +829,19 @@ __device__ bool warp_screen(const double* w, float* wf, const double* __restrict
   using TB = Tab<K>;
   constexpr int N = TB::N;
   const double gm1 = g.gamma - 1.0;
+  const LimUnits un(w[0], w[4 * N]);
   bool bad = false;
   for (int r = lane; r < 5 * N; r += 32) {
     bad |= !finite64(w[r]);
-    wf[r] = f64_to_f32(w[r]);
+    wf[r] = f64_to_f32(exp_add(w[r], un.of(r / N)));
   }
   float* e = wf + 5 * N;  // error bounds of the five values, density threshold
   if (lane < 5) {
     const double* lmax = tab64 + (g.lim_vol ? TB::LMAXV : TB::LMAX);
     double s = fabs(w[lane * N]);
     for (int l = 1; l < N; ++l) s += fabs(w[lane * N + l]) * __ldg(lmax + l);
-    e[lane] = f64_to_f32(2e-6 * s);
-    if (lane == 0) e[5] = f64_to_f32(g.eps_rho * (1.0 + 1e-6) + 1e-5 * s);
+    e[lane] = f64_to_f32(exp_add(2e-6 * s, un.of(lane)));
+    if (lane == 0) e[5] = f64_to_f32(exp_add(g.eps_rho * (1.0 + 1e-6) + 1e-5 * s, un.r));
   }
   // any lane: 1 not finite, 2 some point fails
   unsigned any = bad ? 1u : 0u;
@@ -858,7 +859,8 @@ __device__ bool warp_screen(const double* w, float* wf, const double* __restrict
     return false;
   }
   if (N == 1) return false;
-  const float eps_pf = f64_to_f32(g.eps_p * (1.0 + 1e-6)), gm1f = f64_to_f32(gm1);
+  if (!un.ok) return true;
+  const float eps_pf = f64_to_f32(exp_add(g.eps_p * (1.0 + 1e-6), un.e)), gm1f = f64_to_f32(gm1);
   const int npts = TB::NL + (g.lim_vol ? TB::Q3 : 0);
   for (int s = lane; s < npts; s += 32) {
     const float* ph = s < TB::NL ? tab32 + TB::LPHI + s * N : tab32 + TB::VPHI + (s - TB::NL) * N;

@@ -37,13 +37,15 @@ def driver(k):
     return os.path.join(_dir.name, f"launch_k{k}")
 
 
-def run(k, args, state, outputs):
-    """Run a command with the placeholders "in" (the state, canonical layout)
-    and "out0", "out1", ... replaced by files; the printed values and the
+def run(k, args, state, outputs, modes=None):
+    """Run a command with the placeholders "in" (the state, canonical layout),
+    "modes" and "out0", "out1", ... replaced by files; the printed values and the
     output states in canonical layout."""
     exe = driver(k)
     with tempfile.TemporaryDirectory() as d:
-        path = {"in": os.path.join(d, "in"), **{f"out{j}": os.path.join(d, f"out{j}") for j in range(outputs)}}
+        path = {x: os.path.join(d, x) for x in ("in", "modes", *(f"out{j}" for j in range(outputs)))}
         emu._layout(state).tofile(path["in"])
+        if modes is not None:
+            np.ascontiguousarray(np.concatenate([np.asarray(m, np.float64) for m in modes], axis=1)).tofile(path["modes"])
         info = emu._run(exe, [path.get(a, a) if isinstance(a, str) else a for a in args], d)
         return info, [emu._canonical(np.fromfile(path[f"out{j}"]), state.shape) for j in range(outputs)]
