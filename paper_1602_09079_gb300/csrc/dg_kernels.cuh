@@ -100,6 +100,30 @@ __device__ __forceinline__ bool limiter_screen(const double* mean, const double*
   return plo >= eps_p + 1e-13 * gm1 * (fabs(mean[4]) + sabs[4] + kin);
 }
 
+// The same of a cell whose new coefficients w (rows nc apart) a thread reads back:
+// decides for the cells that an FP32 screen does not clear, so that the FP64
+// path's queue (dg_limiter_counts, the indicator's input) is decided in FP64
+template <int K>
+__device__ bool limiter_screen_of(const double* w, size_t nc, const double* __restrict__ lmax,
+                                               const Geo& g) {
+  constexpr int N = nmodes(K);
+  double m[5], a[5];
+  bool fin = true;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    m[i] = w[(size_t)(i * N) * nc];
+    fin &= finite64(m[i]);
+    a[i] = 0.0;
+#pragma unroll 1
+    for (int l = 1; l < N; ++l) {
+      const double v = w[(size_t)(i * N + l) * nc];
+      a[i] += fabs(v) * __ldg(lmax + l);
+      fin &= finite64(v);
+    }
+  }
+  return limiter_screen<K>(m, a, fin, g.gamma, g.eps_rho, g.eps_p);
+}
+
 // --------------------------------------------------------------- volume
 template <int K, typename T, int MODE, bool FORCE>
 __global__ void __launch_bounds__(kThreads) volume_kernel(const double* __restrict__ yin, const T* __restrict__ fh,
@@ -1505,8 +1529,8 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
     }
   }
   if (MODE == MODE_RHS) return;
-  // limiter screen of the next stage's input (FP32, sufficient); cells that
-  // fail it are queued for the full limiter
+  // limiter screen of the next stage's input: FP32 (sufficient) for all cells,
+  // FP64 for those it does not clear; what fails both is queued for the full limiter
   sScr[(qz * 5 + i) * C + c] = sab * (1.f + 1e-5f);
   __syncthreads();
   if (tid < C && live) {
@@ -1518,7 +1542,8 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
 #pragma unroll
       for (int z = 0; z < Q; ++z) s[v] += sScr[(z * 5 + v) * C + tid];
     }
-    if (!screen_f32(m, s, (float)gm1, (float)g.eps_rho, (float)g.eps_p)) {
+    if (!screen_f32(m, s, (float)gm1, (float)g.eps_rho, (float)g.eps_p) &&
+        !limiter_screen_of<K>(st.out + cell, nc, tab64 + (g.lim_vol ? TB::LMAXV : TB::LMAX), g)) {
       const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
       st.list[slot] = (int)cell;
     }
@@ -2309,9 +2334,9 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
     // the kinetic energy of the means stays: the drop of the internal energy is
     // that of the total
     diss = sM[4 * C + c] - sEn[c];
-    // FP32 screen (the FP64 one took two divisions and some 30 further FP64
+    // FP32 screen first (the FP64 one takes two divisions and some 30 further FP64
     // operations per cell: reset and limiter at 128^3, degree 2, FP32-mixed, 0.41
-    // ms with it, 0.35 so)
+    // ms with it for every cell, 0.35 so)
     float m[5], a[5];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -2321,7 +2346,32 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
     }
     m[4] = f64_to_f32_q(sEn[c]);
     a[4] = sf * (1.f + 1e-5f);
-    if (!fin || !screen_f32(m, a, (float)(g.gamma - 1.0), (float)g.eps_rho, (float)g.eps_p)) {
+    bool queue = !fin || !screen_f32(m, a, (float)(g.gamma - 1.0), (float)g.eps_rho, (float)g.eps_p);
+    if (queue && fin) {
+      // the FP64 test decides, on FP64 sums (mixed: on the FP32 sums, widened)
+      double md[5], ad[5];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) {
+        md[i] = i < 4 ? sM[i * C + c] : sEn[c];
+        if constexpr (sizeof(T) == 8) {
+          ad[i] = 0.0;
+#pragma unroll 1
+          for (int l = 1; l < N; ++l)
+            ad[i] += fabs(i < 4 ? y[(size_t)(i * N + l) * nc + cell] : sEn[l * C + c]) *
+                     __ldg(tab + (g.lim_vol ? TB::LMAXV : TB::LMAX) + l);
+        } else if (i < 4) {
+          ad[i] = sA[i * C + c];
+        } else {
+          float se = 0.f;
+#pragma unroll 1
+          for (int l = 1; l < N; ++l)
+            se += fabsf(f64_to_f32(sEn[l * C + c])) * c_tab32[(g.lim_vol ? TB::LMAXV : TB::LMAX) + l];
+          ad[i] = (double)se * (1.0 + 1e-5);
+        }
+      }
+      queue = !limiter_screen<K>(md, ad, true, g.gamma, g.eps_rho, g.eps_p);
+    }
+    if (queue) {
       const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
       list[slot] = (int)cell;
     }
