@@ -1141,17 +1141,33 @@ struct VolSF {
 // FP64: one (cell, variable, slice of constant z) per thread
 template <int K>
 struct VolSF<K, double> {
-  static constexpr int Q = K + 1, Q3 = Q * Q * Q, N = nmodes(K);
+  static constexpr int Q = K + 1, Q3 = Q * Q * Q, N = nmodes(K), T = (K + 1) * (K + 2) / 2;
+  static constexpr int NL = nmodes(K - 1);  // modes with an exponent above 0 along a given axis
   static constexpr int C = kThreads / (5 * Q);
   // shared memory in doubles: values [5][Q3][C], fluxes and sources [13][Q3][C];
-  // then, over both, the slices' sums [Q][5 N][C] (64-bit integers), their
-  // exponents [Q][5][C] (int), and the screen's [Q + 1][5][C] (float)
-  static constexpr int U = 0, F = 5 * Q3 * C, EXPS = Q * 5 * N * C, SCREEN = EXPS + (Q * 5 * C + 1) / 2;
+  // then, over both, 64-bit integers: the slices' sums of each direction
+  // [Q][3][5][NL][C], their source sums of the modes u = 0 [Q][4][T][C], the faces' sums
+  // [3][5][N][C]; exponents (int) of the slices' [Q][4][5][C] and of the faces'
+  // [3][5][C], and the screen's [Q + 1][5][C] (float)
+  static constexpr int U = 0, F = 5 * Q3 * C;
+  static constexpr int SRC = Q * 15 * NL * C, FACE = SRC + Q * 4 * T * C, EXPS = FACE + 15 * N * C;
+  static constexpr int SCREEN = EXPS + ((Q * 20 + 15) * C + 1) / 2;
   static constexpr int A = 18 * Q3 * C, B = SCREEN + ((Q + 1) * 5 * C + 1) / 2, END = A > B ? A : B;
   static constexpr size_t smem() { return sizeof(double) * END; }
-  // CTAs per SM the register budget is sized for (128 registers)
-  static constexpr int MINB = 2;
+  // CTAs per SM the register budget is sized for (128^3, degree 2: 5.5 ms with 3, 7.1
+  // with 2; degree 3 has no shared memory for a third)
+  static constexpr int MINB = K <= 2 ? 3 : 2;
+  // directions whose faces one slice's threads take
+  static constexpr int NF = (2 + Q) / Q;
 };
+
+// index of the mode with the exponent along an axis lowered by one (255: it is 0)
+static __constant__ unsigned char c_lower[3][20] = {
+    {255, 0, 255, 255, 1, 2, 3, 255, 255, 255, 4, 5, 6, 7, 8, 9, 255, 255, 255, 255},
+    {255, 255, 0, 255, 255, 1, 255, 2, 3, 255, 255, 4, 255, 5, 6, 255, 7, 8, 9, 255},
+    {255, 255, 255, 0, 255, 255, 1, 255, 2, 3, 255, 255, 4, 255, 5, 6, 255, 7, 8, 9}};
+// index among the modes u = 0 (0 for the others); (v, w) has (v + w)(v + w + 1)/2 + w
+static __constant__ unsigned char c_flat[20] = {0, 0, 1, 2, 0, 0, 0, 3, 4, 5, 0, 0, 0, 0, 0, 0, 6, 7, 8, 9};
 
 template <int K>
 __device__ __forceinline__ void pair_uv(int j, int& u, int& v) {
@@ -1175,10 +1191,11 @@ __device__ __forceinline__ void fx_raise(long long (&acc)[N], int& A, int B) {
   }
 }
 
-// acc += the two faces normal to D, from the moments of their fluxes (low face
-// at ml, high face at mh, rows nc apart; face_sf64_kernel): Pt_e(-1) M_low -
-// Pt_e(+1) M_high for the mode e along D, Pt_e(-1) = (-1)^e Pt_e(+1); the
-// moments times inv_dx[D] 2^-p = S 2^-58 (unity: 1)
+// The two faces normal to D of one (cell, variable), from the moments of their
+// fluxes (low face at ml, high face at mh, rows nc apart; face_sf64_kernel):
+// Pt_e(-1) M_low - Pt_e(+1) M_high for the mode e along D, Pt_e(-1) = (-1)^e
+// Pt_e(+1). With the moments' exponent A: the modes e = 0 as M_low - M_high in units
+// of A, exactly 0 where the flow does not change along D; e > 0 divided by 16.
 template <int K, int D>
 __device__ __forceinline__ void fx_apply(const long long (&even)[(K + 1) * (K + 2) / 2],
                                          const long long (&odd)[(K + 1) * (K + 2) / 2],
@@ -1188,25 +1205,19 @@ __device__ __forceinline__ void fx_apply(const long long (&even)[(K + 1) * (K + 
   for (int a = 0, j = 0; a <= K; ++a)
 #pragma unroll
     for (int b = 0; a + b <= K; ++b, ++j) {
-      acc[face_mode<D>(0, a, b)] += even[j] >> 4;  // Pt_0 / 16
+      acc[face_mode<D>(0, a, b)] = even[j];
       const Fx ev = fx_split(even[j]), od = fx_split(odd[j]);
 #pragma unroll
       for (int e = 1; e + a + b <= K; ++e) {
         FxAcc t{0, 0};
         fx_madt(t, e % 2 ? od : ev, F + e);
-        acc[face_mode<D>(e, a, b)] += e % 2 ? -fx_val(t) : fx_val(t);
+        acc[face_mode<D>(e, a, b)] = e % 2 ? -fx_val(t) : fx_val(t);
       }
     }
 }
-__device__ __forceinline__ long long fx_scaled(long long x, bool unity, Fx S) {
-  if (unity) return x;
-  FxAcc t{0, 0};
-  fx_mad(t, fx_split(x), S.h, S.l);
-  return fx_val(t);
-}
 template <int K>
 __device__ __forceinline__ void fx_faces(int d, const double* __restrict__ ml, const double* __restrict__ mh,
-                                         size_t nc, bool unity, Fx S, long long (&acc)[nmodes(K)], int& A, int& top) {
+                                         size_t nc, long long (&acc)[nmodes(K)], int& A) {
   constexpr int T = (K + 1) * (K + 2) / 2;
   double l[T], h[T];
   unsigned mx = 0;
@@ -1216,12 +1227,11 @@ __device__ __forceinline__ void fx_faces(int d, const double* __restrict__ ml, c
     h[j] = __ldg(mh + (size_t)j * nc);
     mx = max(mx, max((unsigned)__double2hiint(l[j]) & 0x7fffffffu, (unsigned)__double2hiint(h[j]) & 0x7fffffffu));
   }
-  top = max(top, bexp(mx));
-  fx_raise(acc, A, bexp(mx) + 1);
+  A = max(kFxTiny, bexp(mx) + 1);
   long long even[T], odd[T];
 #pragma unroll
   for (int j = 0; j < T; ++j) {
-    const long long a = fx_scaled(fx_from(l[j], A), unity, S), b = fx_scaled(fx_from(h[j], A), unity, S);
+    const long long a = fx_from(l[j], A), b = fx_from(h[j], A);
     even[j] = a - b;
     odd[j] = a + b;
   }
@@ -1230,24 +1240,125 @@ __device__ __forceinline__ void fx_faces(int d, const double* __restrict__ ml, c
   else fx_apply<K, 2>(even, odd, acc);
 }
 
+// H[(u, v)] = sums over a slice's points qx + Q qy (rows C apart) of the values f
+// of direction D's flux in units of the exponent A, weighted by D'/8 along D (for z
+// that follows later) and by P' along the others; only the modes that the flux
+// along D contributes to (an exponent above 0 along D) are formed. Rows in pairs +-y.
+// With D = 0 the source fs (SRC and src; exponent As <= A - 2, see volume_sf_kernel)
+// joins H for the modes u > 0, weighted by P' throughout; its modes u = 0 go to H0[v]
+// in units of As.
+template <int K, int D, int C, bool SRC = false>
+__device__ __forceinline__ void fx_slice(const double* f, int A, long long (&H)[(K + 1) * (K + 2) / 2],
+                                         const double* fs = nullptr, bool src = false, int As = 0,
+                                         long long* H0 = nullptr) {
+  using FT = FxTab<K>;
+  constexpr int Q = K + 1, U0 = D == 0 ? 1 : 0, V0 = D == 1 ? 1 : 0, UV = D == 2 ? K - 1 : K;
+  constexpr int TY = D == 1 ? FT::D : FT::W, PY = D == 1 ? 1 : 0;
+  auto row = [&](int qy, long long (&g)[K + 1]) {
+    FxAcc G[K + 1];
+    long long v[Q];
+#pragma unroll
+    for (int u = 0; u <= K; ++u) G[u] = {0, 0};
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = fx_from(f[(q + Q * qy) * C], A);
+    fx_project<K, D == 0>(v, G);
+    if constexpr (SRC)
+      if (src) {
+        const int d = min(A - As, 63);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) v[q] = fx_from(fs[(q + Q * qy) * C], As);
+        FxAcc z{0, 0};
+#pragma unroll
+        for (int r = Q - Q / 2; r < Q; ++r) fx_madt(z, fx_split(v[r] + v[Q - 1 - r]), FT::W + r);
+        if (Q % 2) fx_madt(z, fx_split(v[Q / 2]), FT::W + Q / 2);
+        g[0] = fx_val(z);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) v[q] >>= d;
+        fx_project<K, false>(v, G);
+      }
+#pragma unroll
+    for (int u = U0; u <= K; ++u) g[u] = fx_val(G[u]);
+  };
+#pragma unroll
+  for (int j = 0; j < (K + 1) * (K + 2) / 2; ++j) H[j] = 0;
+  if constexpr (SRC)
+#pragma unroll
+    for (int v = 0; v <= K; ++v) H0[v] = 0;
+  if (Q % 2) {
+    long long g[K + 1];
+    row(Q / 2, g);
+#pragma unroll
+    for (int u = U0; u <= UV; ++u) {
+      const Fx x = fx_split(g[u]);
+#pragma unroll
+      for (int v = PY; u + v <= UV; v += 2) {  // the others' weights are 0 at y = 0
+        FxAcc h{0, 0};
+        fx_madt(h, x, TY + v * Q + Q / 2);
+        H[pair_index(K, u, v)] += fx_val(h);
+      }
+    }
+    if constexpr (SRC)
+      if (src) {
+        const Fx x = fx_split(g[0]);
+#pragma unroll
+        for (int v = 0; v <= K; v += 2) {
+          FxAcc h{0, 0};
+          fx_madt(h, x, FT::W + v * Q + Q / 2);
+          H0[v] += fx_val(h);
+        }
+      }
+  }
+#pragma unroll 1
+  for (int r = Q - Q / 2; r < Q; ++r) {
+    long long a[K + 1], b[K + 1];
+    row(r, a);
+    row(Q - 1 - r, b);
+#pragma unroll
+    for (int u = U0; u <= UV; ++u) {
+      const Fx s = fx_split(a[u] + b[u]), d = fx_split(a[u] - b[u]);
+#pragma unroll
+      for (int v = V0; u + v <= UV; ++v) {
+        FxAcc h{0, 0};
+        fx_madt(h, (v + PY) % 2 ? d : s, TY + v * Q + r);
+        H[pair_index(K, u, v)] += fx_val(h);
+      }
+    }
+    if constexpr (SRC)
+      if (src) {
+        const Fx s = fx_split(a[0] + b[0]), d = fx_split(a[0] - b[0]);
+#pragma unroll
+        for (int v = 0; v <= K; ++v) {
+          FxAcc h{0, 0};
+          fx_madt(h, v % 2 ? d : s, FT::W + v * Q + r);
+          H0[v] += fx_val(h);
+        }
+      }
+  }
+}
+
 // Volume integral, surface integral and stage update, FP64. One (cell,
 // variable, slice of constant z) per thread for the contractions, which run in
 // 64-bit fixed point (dg_common.cuh) with one exponent per variable's
-// coefficients and one, raised as the terms come, for the thread's sums of
-// dw/dt (its slice, and the faces of the directions z, z + Q, ...); one (cell,
+// coefficients and one per direction of the fluxes and for the source; one (cell,
 // point) per thread for the Euler fluxes and the driving source, in FP64; then
 // one (cell, variable) and every Q-th mode per thread for the sum over the
-// slices and the stage update. Everything enters the sums as
-//   dw/dt = 2^(p + 4) [sum_d s_d sum_q F_d(q) (D'/8) P' P' + sum_faces +- s_d
-//           (P' P' moments) Pt_e / 16 + sum_q 2^-(p+4) S(q) P' P' P'],
+// slices and the stage update:
+//   dw/dt = sum_d 1/dx_d [16 (sum_q F_d(q) (D'/8) P' P' + sum_faces +- (P' P'
+//           moments) Pt_e / 16)] + 1/dx_x [16 sum_q (dx_x / 16) S(q) P' P' P'],
 // P' = P w / 2 and D' = (dP/dxi) w / 2 (sums of |P'| <= 1, of |D'| / 8 <= 0.61),
-// 2^p >= 1/dx_d = s_d 2^p. Inputs take 60 bits and the source 58, so that no
-// intermediate reaches 2^61 and no sum 2^63. Integer issue bounds it on large
-// meshes (128^3, degree 2: 7.7 ms per stage, the FP64 contractions took 33.6;
-// 64^3, degree 3: 2.2 ms) and one thread's chain on small ones, which is why a
-// slice is a thread's work: with a thread per (cell, variable) 128^3 took 7.1
-// ms, but 8 x 8 x 8 at degree 1 or 33 x 32 x 31 fill the chip with three or
-// four times the threads (8^3: 11 us, the dense kernel took 84).
+// the bracket of a direction in fixed point, the brackets added in FP64: a direction
+// whose fluxes are far above another's contributes exactly 0 to the modes constant
+// along it where the flow does not change along it, and must not cut the other's
+// terms. The source joins the x flux in the modes that this contributes to and has
+// an exponent of its own in the others. Inputs take 60 bits and the source there 58,
+// so that no intermediate reaches 2^61 and no sum 2^63. Integer issue bounds it on large
+// meshes (128^3, degree 2: 5.5 ms per stage, 7.1 with driving; with one exponent for
+// the three directions and the source, two CTAs per SM, 6.9 and 7.6, with FP64
+// contractions 33.6; 64^3, degree 3: 2.28 and 2.67, before 2.16 and 2.61) and one
+// thread's chain on small ones, which is why a slice is a thread's work: a thread per
+// (cell, variable) was 7 % faster at 128^3, but 8 x 8 x 8 at degree 1 or 33 x 32 x 31
+// fill the chip with three or four times the threads (8^3: 12 us, the dense kernel
+// took 84).
 template <int K, typename T, int MODE, bool FORCE>
 __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
     volume_sf_kernel(const double* __restrict__ yin, const float* __restrict__ yf32, const T* __restrict__ fh,
@@ -1258,7 +1369,7 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
   using TB = Tab<K>;
   using CF = VolSF<K, double>;
   using FT = FxTab<K>;
-  constexpr int N = TB::N, Q = K + 1, Q2 = Q * Q, Q3 = TB::Q3, C = CF::C, T2 = (K + 1) * (K + 2) / 2;
+  constexpr int N = TB::N, Q = K + 1, Q2 = Q * Q, Q3 = TB::Q3, C = CF::C, T2 = CF::T, NL = CF::NL;
   static_assert(kThreads == 5 * Q * C, "one (cell, variable, slice) per thread");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* sm64 = reinterpret_cast<double*>(smem_raw);
@@ -1271,13 +1382,13 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
   const bool live = cell < nc;
   const long long cellc = live ? cell : nc - 1;  // ragged tail: in-bounds reads, nothing written
   const double* ysrc = (MODE == MODE_STAGE) ? st.ys : yin;
-  int top = 0;  // largest exponent seen
+  bool huge = false;  // values or fluxes that have no exponent (kFxHuge): the result is NaN
   // --------------------------------------------- values at the slice's points
   {
     Fx x[N];
     int B;
     fx_load<K>(ysrc + (size_t)(i * N) * nc + cellc, nc, x, B);
-    if (B >= kFxHuge) top = kFxHuge;
+    huge = B >= kFxHuge;
     Fx pz[K + 1];  // Pt_w at the slice
 #pragma unroll
     for (int ww = 1; ww <= K; ++ww) pz[ww] = {c_fx[FT::P + ww * Q + qz][0], c_fx[FT::P + ww * Q + qz][1]};
@@ -1303,24 +1414,19 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
       for (int qx = 0; qx < Q; ++qx) u[(qx + Q * qy) * C] = fx_to_double(v[qx], B);
     }
   }
-  // 2^p >= every 1/dx; s_d = 1/dx_d 2^-p as a multiplier S 2^-58 (1: skipped)
-  const double im = fmax(g.inv_dx[0], fmax(g.inv_dx[1], g.inv_dx[2]));
-  const int pb = bexp((unsigned)__double2hiint(im)) + ((__double_as_longlong(im) & 0xfffffffffffffLL) ? 1 : 0);
-  const int p4 = pb - 1023 + 4;
-  const double unit = __hiloint2double(pb << 20, 0);
-  long long acc[N];
-#pragma unroll
-  for (int l = 0; l < N; ++l) acc[l] = 0;
-  int A = kFxTiny;
+  // the faces of the directions qz, qz + Q, ...
+  long long facc[CF::NF][N];
+  int fexp[CF::NF];
   {
     int ix, iy, iz;
     cell_xyz(cellc, g, ix, iy, iz);
-#pragma unroll 1
-    for (int d = qz; d < 3; d += Q) {
-      const double* f = fh + (size_t)((d * 5 + i) * T2) * nc;
-      const double idx = d == 0 ? g.inv_dx[0] : (d == 1 ? g.inv_dx[1] : g.inv_dx[2]);
-      fx_faces<K>(d, f + cellc, f + neighbour(g, ix, iy, iz, d, 1), nc, idx == unit, fx_split(fx_from(idx, pb) >> 2),
-                  acc, A, top);
+#pragma unroll
+    for (int n = 0; n < CF::NF; ++n) {
+      const int d = qz + n * Q;
+      if (d < 3) {
+        const double* f = fh + (size_t)((d * 5 + i) * T2) * nc;
+        fx_faces<K>(d, f + cellc, f + neighbour(g, ix, iy, iz, d, 1), nc, facc[n], fexp[n]);
+      }
     }
   }
   __syncthreads();
@@ -1337,7 +1443,7 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
         const int q = it / C, cc = it % C;
         const T* ap = field + (size_t)q * nc + (c0 + cc < nc ? c0 + cc : nc - 1);
 #pragma unroll
-        for (int d = 0; d < 3; ++d) a[d] = __ldg(ap + (size_t)d * Q3 * nc);
+        for (int d = 0; d < 3; ++d) a[d] = 0.0625 * g.dx[0] * __ldg(ap + (size_t)d * Q3 * nc);
       }
       const double r = sU[it], m0 = sU[R3 + it], m1 = sU[2 * R3 + it], m2 = sU[3 * R3 + it], E = sU[4 * R3 + it];
       const double ir = rcp64(r);
@@ -1363,6 +1469,10 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
   }
   __syncthreads();
   // -------------------- projection onto the basis gradients (and the source)
+  const bool src = FORCE && i > 0;
+  // by direction, modes by their index with the exponent along it lowered by one
+  long long V[3][NL], S[FORCE ? T2 : 1];  // S: the source's modes (0, v, w)
+  int ex[3], es = kFxTiny;
   {
     // where this variable's fluxes along x, y, z and its source lie: the mass
     // flux is the momentum itself, the momentum flux is symmetric
@@ -1373,122 +1483,74 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
       fd[d] = (i == 0 ? sm64 + CF::U + (1 + d) * Q3 * C : sm64 + CF::F + (i == 4 ? 6 + d : sym[d]) * Q3 * C) +
               qz * Q2 * C + c;
     const double* fs = sm64 + CF::F + ((9 + (i > 0 ? i - 1 : 0)) * Q3 + qz * Q2) * C + c;
-    const bool src = FORCE && i > 0;
-    bool one[3];
-    Fx S[3];
+    unsigned mx[3] = {0, 0, 0}, ms = 0;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      one[d] = g.inv_dx[d] == unit;
-      S[d] = fx_split(fx_from(g.inv_dx[d], pb) >> 2);
+    for (int q = 0; q < Q2; ++q) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) mx[d] = max(mx[d], (unsigned)__double2hiint(fd[d][q * C]) & 0x7fffffffu);
+      if (src) ms = max(ms, (unsigned)__double2hiint(fs[q * C]) & 0x7fffffffu);
     }
-    unsigned mx = 0, ms = 0;
 #pragma unroll
-      for (int q = 0; q < Q2; ++q) {
+    for (int d = 0; d < 3; ++d) ex[d] = max(kFxTiny, bexp(mx[d]) + 1);
+    long long H[T2];
+    if constexpr (FORCE) {
+      es = max(kFxTiny, bexp(ms) + 1);
+      if (src) ex[0] = max(ex[0], es + 2);
+      long long H0[K + 1];
+      fx_slice<K, 0, C, true>(fd[0], ex[0], H, fs, src, es, H0);
+      if (src) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) mx = max(mx, (unsigned)__double2hiint(fd[d][q * C]) & 0x7fffffffu);
-        if (src) ms = max(ms, (unsigned)__double2hiint(fs[q * C]) & 0x7fffffffu);
-      }
-      top = max(top, max(bexp(mx), bexp(ms)));
-      fx_raise(acc, A, max(bexp(mx) + 1, ms ? bexp(ms) - p4 + 3 : 0));
-      // rows of constant y: Gx, Gy, Gz = sums along x
-      auto row = [&](int qy, long long (&gx)[K + 1], long long (&gy)[K + 1], long long (&gz)[K + 1]) {
-        FxAcc G[K + 1];
-        long long f[Q];
+        for (int ww = 0; ww <= K; ++ww) {
+          const int h = c_fx[FT::W + ww * Q + qz][0], l = c_fx[FT::W + ww * Q + qz][1];
 #pragma unroll
-        for (int u = 0; u <= K; ++u) G[u] = {0, 0};
-#pragma unroll
-        for (int q = 0; q < Q; ++q) f[q] = fx_scaled(fx_from(fd[0][(q + Q * qy) * C], A), one[0], S[0]);
-        fx_project<K, true>(f, G);
-        if (src) {
-          // weighted by P' along all three axes, like the x flux along y and
-          // z: it joins the x flux's sums here
-#pragma unroll
-          for (int q = 0; q < Q; ++q) f[q] = fx_from(fs[(q + Q * qy) * C], A + p4);
-          fx_project<K, false>(f, G);
-        }
-#pragma unroll
-        for (int u = 0; u <= K; ++u) {
-          gx[u] = fx_val(G[u]);
-          G[u] = {0, 0};
-        }
-#pragma unroll
-        for (int q = 0; q < Q; ++q) f[q] = fx_scaled(fx_from(fd[1][(q + Q * qy) * C], A), one[1], S[1]);
-        fx_project<K, false>(f, G);
-#pragma unroll
-        for (int u = 0; u <= K; ++u) {
-          gy[u] = fx_val(G[u]);
-          G[u] = {0, 0};
-        }
-#pragma unroll
-        for (int q = 0; q < Q; ++q) f[q] = fx_scaled(fx_from(fd[2][(q + Q * qy) * C], A), one[2], S[2]);
-        fx_project<K, false>(f, G);
-#pragma unroll
-        for (int u = 0; u <= K; ++u) gz[u] = fx_val(G[u]);
-      };
-      // H1 = sum over y of Gx P' + Gy D', H2 = of Gz P', by pairs of rows
-      long long H1[T2], H2[T2];
-#pragma unroll
-      for (int j = 0; j < T2; ++j) H1[j] = H2[j] = 0;
-      if (Q % 2) {
-        long long gx[K + 1], gy[K + 1], gz[K + 1];
-        row(Q / 2, gx, gy, gz);
-#pragma unroll
-        for (int u = 0, j = 0; u <= K; ++u) {
-          const Fx x = fx_split(gx[u]), yy = fx_split(gy[u]), z = fx_split(gz[u]);
-#pragma unroll
-          for (int v = 0; u + v <= K; ++v, ++j) {
-            FxAcc h1{0, 0}, h2{0, 0};
-            if (v % 2 == 0) {
-              fx_madt(h1, x, FT::W + v * Q + Q / 2);
-              fx_madt(h2, z, FT::W + v * Q + Q / 2);
-              H2[j] += fx_val(h2);
-            } else {
-              fx_madt(h1, yy, FT::D + v * Q + Q / 2);
-            }
-            H1[j] += fx_val(h1);
-          }
-        }
-      }
-#pragma unroll 1
-      for (int r = Q - Q / 2; r < Q; ++r) {
-        long long ax[K + 1], ay[K + 1], az[K + 1], bx[K + 1], by[K + 1], bz[K + 1];
-        row(r, ax, ay, az);
-        row(Q - 1 - r, bx, by, bz);
-#pragma unroll
-        for (int u = 0, j = 0; u <= K; ++u) {
-          const Fx xs = fx_split(ax[u] + bx[u]), xd = fx_split(ax[u] - bx[u]);
-          const Fx ys_ = fx_split(ay[u] + by[u]), yd = fx_split(ay[u] - by[u]);
-          const Fx zs = fx_split(az[u] + bz[u]), zd = fx_split(az[u] - bz[u]);
-#pragma unroll
-          for (int v = 0; u + v <= K; ++v, ++j) {
-            FxAcc h1{0, 0}, h2{0, 0};
-            fx_madt(h1, v % 2 ? xd : xs, FT::W + v * Q + r);
-            if (v > 0) fx_madt(h1, v % 2 ? ys_ : yd, FT::D + v * Q + r);
-            fx_madt(h2, v % 2 ? zd : zs, FT::W + v * Q + r);
-            H1[j] += fx_val(h1);
-            H2[j] += fx_val(h2);
-          }
-        }
-      }
-      Fx wz[K + 1], dz[K + 1];
-#pragma unroll
-      for (int ww = 0; ww <= K; ++ww) {
-        wz[ww] = {c_fx[FT::W + ww * Q + qz][0], c_fx[FT::W + ww * Q + qz][1]};
-        dz[ww] = {c_fx[FT::D + ww * Q + qz][0], c_fx[FT::D + ww * Q + qz][1]};
-      }
-#pragma unroll
-      for (int u = 0, j = 0; u <= K; ++u)
-#pragma unroll
-        for (int v = 0; u + v <= K; ++v, ++j) {
-          const Fx h1 = fx_split(H1[j]), h2 = fx_split(H2[j]);
-#pragma unroll
-          for (int ww = 0; u + v + ww <= K; ++ww) {
+          for (int v = 0; v + ww <= K; ++v) {
             FxAcc t{0, 0};
-            fx_mad(t, h1, wz[ww].h, wz[ww].l);
-            if (ww > 0) fx_mad(t, h2, dz[ww].h, dz[ww].l);
-            acc[mode_index(u, v, ww)] += fx_val(t);
+            fx_mad(t, fx_split(H0[v]), h, l);
+            S[(v + ww) * (v + ww + 1) / 2 + ww] = fx_val(t);
           }
         }
+      }
+    } else {
+      fx_slice<K, 0, C>(fd[0], ex[0], H);
+    }
+#pragma unroll
+    for (int ww = 0; ww <= K; ++ww) {
+      const int h = c_fx[FT::W + ww * Q + qz][0], l = c_fx[FT::W + ww * Q + qz][1];
+#pragma unroll
+      for (int u = 1; u + ww <= K; ++u)
+#pragma unroll
+        for (int v = 0; u + v + ww <= K; ++v) {
+          FxAcc t{0, 0};
+          fx_mad(t, fx_split(H[pair_index(K, u, v)]), h, l);
+          V[0][mode_index(u - 1, v, ww)] = fx_val(t);
+        }
+    }
+    fx_slice<K, 1, C>(fd[1], ex[1], H);
+#pragma unroll
+    for (int ww = 0; ww <= K; ++ww) {
+      const int h = c_fx[FT::W + ww * Q + qz][0], l = c_fx[FT::W + ww * Q + qz][1];
+#pragma unroll
+      for (int u = 0; u + ww <= K; ++u)
+#pragma unroll
+        for (int v = 1; u + v + ww <= K; ++v) {
+          FxAcc t{0, 0};
+          fx_mad(t, fx_split(H[pair_index(K, u, v)]), h, l);
+          V[1][mode_index(u, v - 1, ww)] = fx_val(t);
+        }
+    }
+    fx_slice<K, 2, C>(fd[2], ex[2], H);
+#pragma unroll
+    for (int ww = 1; ww <= K; ++ww) {
+      const int h = c_fx[FT::D + ww * Q + qz][0], l = c_fx[FT::D + ww * Q + qz][1];
+#pragma unroll
+      for (int u = 0; u + ww <= K; ++u)
+#pragma unroll
+        for (int v = 0; u + v + ww <= K; ++v) {
+          FxAcc t{0, 0};
+          fx_mad(t, fx_split(H[pair_index(K, u, v)]), h, l);
+          V[2][mode_index(u, v, ww - 1)] = fx_val(t);
+        }
+    }
   }
   __syncthreads();
   // ------------------------- sum over the slices; R, or the FP64 stage update
@@ -1496,26 +1558,79 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
   int* sExp = reinterpret_cast<int*>(sm64 + CF::EXPS);
   float* sScr = reinterpret_cast<float*>(sm64 + CF::SCREEN);
 #pragma unroll
-  for (int l = 0; l < N; ++l) sAcc[((qz * 5 + i) * N + l) * C + c] = acc[l];
-  sExp[(qz * 5 + i) * C + c] = top >= kFxHuge ? 2 * kFxHuge : A;
-  __syncthreads();
-  int sh[Q], Am = 0;
+  for (int d = 0; d < 3; ++d) {
 #pragma unroll
-  for (int z = 0; z < Q; ++z) {
-    sh[z] = sExp[(z * 5 + i) * C + c];
-    Am = max(Am, sh[z]);
+    for (int m = 0; m < NL; ++m) sAcc[(((qz * 3 + d) * 5 + i) * NL + m) * C + c] = V[d][m];
+    sExp[((qz * 4 + d) * 5 + i) * C + c] = huge ? kFxHuge : ex[d];
   }
+  if constexpr (FORCE)
+    if (src) {
 #pragma unroll
-  for (int z = 0; z < Q; ++z) sh[z] = min(Am - sh[z], 63);
+      for (int j = 0; j < T2; ++j) sAcc[CF::SRC + ((qz * 4 + i - 1) * T2 + j) * C + c] = S[j];
+      sExp[((qz * 4 + 3) * 5 + i) * C + c] = es;
+    }
+#pragma unroll
+  for (int n = 0; n < CF::NF; ++n) {
+    const int d = qz + n * Q;
+    if (d < 3) {
+#pragma unroll
+      for (int l = 0; l < N; ++l) sAcc[CF::FACE + ((d * 5 + i) * N + l) * C + c] = facc[n][l];
+      sExp[((Q * 4 + d) * 5 + i) * C + c] = fexp[n];
+    }
+  }
+  __syncthreads();
+  // per direction: the largest exponent and the shifts to it of the slices (and,
+  // last, of the faces); per slice that of the source
+  int xm[3], fe[3], sh[3][Q + 1], xs = 0, shs[Q], top = 0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    xm[d] = 0;
+#pragma unroll
+    for (int z = 0; z <= Q; ++z) {
+      sh[d][z] = sExp[((z * 4 + d) * 5 + i) * C + c];
+      xm[d] = max(xm[d], sh[d][z]);
+    }
+    fe[d] = sh[d][Q];
+#pragma unroll
+    for (int z = 0; z <= Q; ++z) sh[d][z] = min(xm[d] - sh[d][z], 63);
+    top = max(top, xm[d]);
+  }
+  if (src) {
+#pragma unroll
+    for (int z = 0; z < Q; ++z) {
+      shs[z] = sExp[((z * 4 + 3) * 5 + i) * C + c];
+      xs = max(xs, shs[z]);
+    }
+#pragma unroll
+    for (int z = 0; z < Q; ++z) shs[z] = min(xs - shs[z], 63);
+    top = max(top, xs);
+  }
   float sab = 0.f;
   if (live) {
 #pragma unroll 1
     for (int l = qz; l < N; l += Q) {
       const size_t at = (size_t)(i * N + l) * nc + cell;
-      long long s = 0;
+      double a = 0.0;
 #pragma unroll
-      for (int z = 0; z < Q; ++z) s += sAcc[((z * 5 + i) * N + l) * C + c] >> sh[z];
-      const double a = Am < kFxHuge ? fx_to_double(s, Am + p4) : __longlong_as_double(0x7ff8000000000000LL);
+      for (int d = 0; d < 3; ++d) {
+        const int low = c_lower[d][l];
+        long long t = sAcc[CF::FACE + ((d * 5 + i) * N + l) * C + c];
+        int x = fe[d];  // e = 0: the faces' difference in their own units
+        if (low != 255) {
+          t >>= sh[d][Q];
+#pragma unroll
+          for (int z = 0; z < Q; ++z) t += sAcc[(((z * 3 + d) * 5 + i) * NL + low) * C + c] >> sh[d][z];
+          x = xm[d] + 4;
+        }
+        a = fma(g.inv_dx[d], fx_to_double(t, x), a);
+      }
+      if (src && c_lower[0][l] == 255) {
+        long long t = 0;
+#pragma unroll
+        for (int z = 0; z < Q; ++z) t += sAcc[CF::SRC + ((z * 4 + i - 1) * T2 + c_flat[l]) * C + c] >> shs[z];
+        a = fma(g.inv_dx[0], fx_to_double(t, xs + 4), a);
+      }
+      if (top >= kFxHuge) a = __longlong_as_double(0x7ff8000000000000LL);
       if (MODE == MODE_RHS) {
         R[at] = -a;
       } else {
