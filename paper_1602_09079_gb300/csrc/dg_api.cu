@@ -344,7 +344,6 @@ struct dg_ctx {
   Ctrl* ctrl = nullptr;
   double* part = nullptr;
   double* modes_dev = nullptr;
-  int cfl_slot = 0;            // which of the control block's CFL maxima the next reduction uses
   bool queue_open = false;     // n_flag may not be 0 (see open_queue)
   double* ybuf = nullptr;
   int* list = nullptr;
@@ -681,7 +680,6 @@ int dg_bind(dg_ctx* c, double* y_dev, void* scratch_dev, size_t scratch_bytes, v
   c->ctrl = reinterpret_cast<Ctrl*>(c->scratch + L.ctrl);
   c->part = reinterpret_cast<double*>(c->scratch + L.part);
   c->modes_dev = reinterpret_cast<double*>(c->scratch + L.modes);
-  c->cfl_slot = 0;
   c->queue_open = false;
   c->ybuf = reinterpret_cast<double*>(c->scratch + L.ybuf);
   c->list = reinterpret_cast<int*>(c->scratch + L.list);
@@ -890,14 +888,15 @@ int dg_cfl_dt(dg_ctx* c, double courant, double* dt_out) {
   DG_TRY(need_bound(c));
   if (!dt_out || !(courant > 0.0)) return DG_ERR_ARG;
   DG_TRY(set_device(c));
-  const int slot = c->cfl_slot;
-  c->cfl_slot ^= 1;
-  DG_TRY(launch(c, KC_CFL, [&] { return c->fn.cfl(c->y, c->geo, c->ctrl, slot, c->stream); }));
+  // cleared by every call: nothing is left over from a reduction that was not
+  // launched, or from another context that uses this scratch in turn
+  DG_CUDA(cudaMemsetAsync(&c->ctrl->cfl_max_bits, 0, sizeof(unsigned long long), c->stream));
+  DG_TRY(launch(c, KC_CFL, [&] { return c->fn.cfl(c->y, c->geo, c->ctrl, c->stream); }));
   Ctrl h{};
   int st = sync_and_check(c, &h);
   if (st != DG_OK) return st;
   double smax;
-  std::memcpy(&smax, slot ? &h.cfl_max_bits2 : &h.cfl_max_bits, sizeof(double));
+  std::memcpy(&smax, &h.cfl_max_bits, sizeof(double));
   if (!(smax > 0.0)) return DG_ERR_POSITIVITY;
   // C min(1/(2k+1), w1/2) with w1 = 1 (m = 2 GLL points), 1/3 (m = 3)
   const double w1 = gll_m(c->k) == 2 ? 1.0 : 1.0 / 3.0;

@@ -141,7 +141,6 @@ struct Ctrl {
   unsigned int n_deep;              // queued cells the FP32 point screen does not clear
   unsigned long long n_queued_total;  // cells that failed the limiter screen (all stages)
   unsigned long long n_full_total;    // cells that went through the full limiter
-  unsigned long long cfl_max_bits2;   // the maximum of every second CFL reduction; each clears the other's
   double sums[8];                     // results of the host-facing sums, read back with the error word
 };
 

@@ -244,8 +244,8 @@ cudaError_t limit(double* y, int8_t* flags, const Geo& g, Ctrl* ctrl, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t cfl(const double* y, const Geo& g, Ctrl* ctrl, int slot, cudaStream_t s) {
-  return launch_after(cfl_kernel<KK>, grid1(g.nc, kCflThreads), kCflThreads, 0, s, y, g, ctrl, slot);
+cudaError_t cfl(const double* y, const Geo& g, Ctrl* ctrl, cudaStream_t s) {
+  return launch_after(cfl_kernel<KK>, grid1(g.nc, kCflThreads), kCflThreads, 0, s, y, g, ctrl);
 }
 
 template <typename T>

@@ -2030,12 +2030,9 @@ __global__ void __launch_bounds__(kThreads) limit_kernel(double* __restrict__ y,
 constexpr int kCflThreads = 256;
 
 template <int K>
-__global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restrict__ y, Geo g, Ctrl* ctrl,
-                                                          int slot = 0) {
+__global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restrict__ y, Geo g, Ctrl* ctrl) {
   stream_wait();
   constexpr int N = nmodes(K);
-  unsigned long long* const max_bits = slot ? &ctrl->cfl_max_bits2 : &ctrl->cfl_max_bits;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *(slot ? &ctrl->cfl_max_bits : &ctrl->cfl_max_bits2) = 0ull;
   const long long nc = g.nc;
   const long long c = (long long)blockIdx.x * kCflThreads + threadIdx.x;
   double r = 1.0, m1 = 0.0, m2 = 0.0, m3 = 0.0, E = 0.0;
@@ -2101,7 +2098,7 @@ __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restri
       if (u > v) v = u;
     }
     if (threadIdx.x == 0) {
-      atomicMax(max_bits, v);
+      atomicMax(&ctrl->cfl_max_bits, v);
       if (s_err) atomicOr(&ctrl->err, s_err);
     }
   }

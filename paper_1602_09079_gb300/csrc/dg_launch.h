@@ -42,9 +42,8 @@ struct Launchers {
   // screen[c] = 1 if cell c fails the limiter screen
   cudaError_t (*screen)(const double* y, uint8_t* screen, const Geo& g, cudaStream_t s);
   cudaError_t (*limit)(double* y, int8_t* flags, const Geo& g, Ctrl* ctrl, cudaStream_t s);
-  // slot: which of the control block's two maxima to use (zero on entry; the
-  // other one is cleared)
-  cudaError_t (*cfl)(const double* y, const Geo& g, Ctrl* ctrl, int slot, cudaStream_t s);
+  // into ctrl->cfl_max_bits (0 on entry)
+  cudaError_t (*cfl)(const double* y, const Geo& g, Ctrl* ctrl, cudaStream_t s);
   // returns the number of partial sums written to part; cells failing the
   // limiter screen afterwards are queued in list / ctrl->n_flag (0 on entry)
   cudaError_t (*energy_reset)(int prec, double* y, const Geo& g, double c2g, double inv_rho0, double* part,
