@@ -344,7 +344,6 @@ struct dg_ctx {
   Ctrl* ctrl = nullptr;
   double* part = nullptr;
   double* modes_dev = nullptr;
-  bool queue_open = false;     // n_flag may not be 0 (see open_queue)
   double* ybuf = nullptr;
   int* list = nullptr;
   int* list2 = nullptr;
@@ -445,12 +444,12 @@ int sync_and_check(dg_ctx* c, Ctrl* host_copy) {
   return err_to_status(h.err);
 }
 
-// Cells are about to be queued: the queue is empty unless an earlier call
-// failed between the kernel that queued cells and the limiter that empties it.
-int open_queue(dg_ctx* c) {
-  if (c->queue_open) DG_CUDA(cudaMemsetAsync(&c->ctrl->n_flag, 0, sizeof(unsigned), c->stream));
-  c->queue_open = true;
-  return DG_OK;
+// Empties the limiter's queue: the first thing in a call that queues cells, whatever
+// an earlier call (of this context, or of another one on the same scratch) has left
+// there. Between the stages of a call the limiter's last pass leaves it empty; the
+// unfused stages' face kernels empty it themselves.
+int empty_queue(dg_ctx* c) {
+  return cuda_ok(cudaMemsetAsync(&c->ctrl->n_flag, 0, sizeof(unsigned), c->stream));
 }
 
 int set_device(const dg_ctx* c) { return cuda_ok(cudaSetDevice(c->device)); }
@@ -558,7 +557,7 @@ int fused_step(dg_ctx* c, double dt, bool force) {
     a.b0_d = b0[s];
     a.y0 = c->y;
     a.stage = s + 1;
-    DG_TRY(open_queue(c));
+    if (s == 0) DG_TRY(empty_queue(c));
     DG_TRY(launch(c, KC_VOLUME, [&] { return c->fz.run(force, c->flux, c->geo, a, c->stream); }));
     float* yf = s == 2 ? c->yf : nullptr;
     const double* y0 = s < 2 ? c->y : nullptr;
@@ -579,7 +578,6 @@ int fused_step(dg_ctx* c, double dt, bool force) {
                                 c->stream);
       }, 2));
     }
-    c->queue_open = false;
     ys = out;
   }
   c->limited = true;
@@ -680,7 +678,6 @@ int dg_bind(dg_ctx* c, double* y_dev, void* scratch_dev, size_t scratch_bytes, v
   c->ctrl = reinterpret_cast<Ctrl*>(c->scratch + L.ctrl);
   c->part = reinterpret_cast<double*>(c->scratch + L.part);
   c->modes_dev = reinterpret_cast<double*>(c->scratch + L.modes);
-  c->queue_open = false;
   c->ybuf = reinterpret_cast<double*>(c->scratch + L.ybuf);
   c->list = reinterpret_cast<int*>(c->scratch + L.list);
   c->list2 = reinterpret_cast<int*>(c->scratch + L.list2);
@@ -837,7 +834,6 @@ int dg_step(dg_ctx* c, double dt) {
   for (int s = 0; s < 3; ++s) {
     double* out = s < 2 ? c->ybuf : c->y;
     DG_TRY(launch(c, KC_FACE, [&] { return c->fn.face(c->prec, c->flux, ys, yf, c->fh, c->geo, c->ctrl, c->stream); }));
-    DG_TRY(open_queue(c));
     DG_TRY(launch(c, KC_VOLUME, [&] {
       return c->fn.volume_stage(c->prec, force, c->fh, c->field, c->geo, ys, c->y, out, a0[s], b0[s], dt, c->list,
                                 yf, c->ctrl, c->stream);
@@ -860,7 +856,6 @@ int dg_step(dg_ctx* c, double dt) {
                                 c->stream);
       }, 2));
     }
-    c->queue_open = false;
     ys = out;
   }
   c->limited = true;
@@ -971,7 +966,7 @@ int dg_energy_reset(dg_ctx* c, double c_iso, double rho0, double* dissipated) {
   // keep the FP32 shadow current if it is (energy rows and limited cells)
   float* yf = (uses_shadow(c) && c->shadow_valid) ? c->yf : nullptr;
   if (!yf) c->shadow_valid = false;
-  DG_TRY(open_queue(c));
+  DG_TRY(empty_queue(c));
   DG_TRY(launch(c, KC_RESET, [&] {
     return c->fn.energy_reset(c->prec, c->y, c->geo, c2g, 1.0 / rho0, c->part, &n_part, c->list, c->ctrl, yf,
                               c->stream);
@@ -982,7 +977,6 @@ int dg_energy_reset(dg_ctx* c, double c_iso, double rho0, double* dissipated) {
     return c->fn.limit_list(c->y, c->list, &c->ctrl->n_flag, c->geo, c->ctrl, 0, yf, nullptr, nullptr, c->list2,
                                 c->stream);
   }, 2));
-  c->queue_open = false;
   c->limited = true;
   if (dissipated) {
     const double vol = c->geo.dx[0] * c->geo.dx[1] * c->geo.dx[2];

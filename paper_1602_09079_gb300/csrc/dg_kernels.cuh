@@ -49,6 +49,11 @@ struct StageArgs {
                      // this CTA's cells, then overwritten with the output
 };
 
+// the queue's counter, by the face kernels: the volume kernel after them queues cells
+__device__ __forceinline__ void clear_queue(Ctrl* ctrl) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) ctrl->n_flag = 0u;
+}
+
 // first thing in every kernel that queues cells: the second pass's counter
 __device__ __forceinline__ void clear_deep(Ctrl* ctrl) {
   if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->n_deep = 0u;
@@ -491,6 +496,7 @@ __global__ void __launch_bounds__(FaceSF64<K>::THREADS, FaceSF64<K>::MINB) face_
   double* sU = reinterpret_cast<double*>(smem_raw);
   const long long nc = g.nc, c0 = (long long)blockIdx.x * C;
   const int c = threadIdx.x % C, i = threadIdx.x / C;  // i: conserved variable, warp-uniform
+  clear_queue(ctrl);
   const long long cell = c0 + c;
   const bool live = cell < nc;
   int ix = 0, iy = 0, iz = 0;
@@ -561,6 +567,7 @@ template <int K, int FLUX>
 __global__ void __launch_bounds__(96, FaceF32<K>::MINB) face_flux_f32_kernel(const float* __restrict__ yf, float* __restrict__ fh,
                                                               Geo g, Ctrl* ctrl) {
   stream_wait();
+  clear_queue(ctrl);
   const long long c = (long long)blockIdx.x * 32 + (threadIdx.x & 31);
   if (c >= g.nc) return;
   const int d = threadIdx.x >> 5;  // warp-uniform direction

@@ -1,6 +1,9 @@
 """Contexts that use one scratch buffer in turn: the scratch holds no result of an
 earlier call that a later one of the other context depends on. dg_cfl_dt of a slow
-flow after that of a fast one (and back) gives what each gives on its own scratch."""
+flow after that of a fast one (and back) gives what each gives on its own scratch. A
+count that a failed call of another context has left in the limiter's queue (the
+control block's fourth word) changes nothing."""
+import numpy as np
 import pytest
 
 import oracle
@@ -37,3 +40,28 @@ def test_cfl_in_turn(dg, order):
         bind(dg, s, solvers[0].scratch)
     for j in (0, 1, 1, 0, 1, 0, 0, 1):
         assert solvers[j].cfl_dt(0.3) == own[j]
+
+
+@pytest.mark.parametrize("order", [1, 2, 3, 4])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_left_over_queue_count(dg, order, mixed):
+    import torch
+    w = syn.random_state(N_MESH, oracle.nmodes(order - 1), syn.GAMMA, seed=9, high=0.2)
+
+    def run(left):
+        s = dg.Solver(N_MESH, order, syn.GAMMA)
+        if mixed:
+            s.set_precision(dg.DG_PREC_MIXED)
+        s.set_state(w)
+        s.step(1e-3)  # the queue's list holds cells from here on
+        word = s.scratch[:16].view(torch.int32)
+        for call in (lambda: s.step(1e-3), lambda: s.energy_reset(0.7, 1.0)):
+            assert int(word[3]) == 0
+            word[3] = left
+            call()
+        s.check()
+        return s.get_state(), dg.dg_limiter_counts(s.ctx)
+
+    (a, na), (b, nb) = run(0), run(5)
+    np.testing.assert_array_equal(a, b)
+    assert na == nb
