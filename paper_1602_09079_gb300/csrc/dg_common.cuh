@@ -5,6 +5,13 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+// a device function that is called, not inlined (no such keyword in host builds)
+#ifdef __CUDACC__
+#define DG_NOINLINE __noinline__
+#else
+#define DG_NOINLINE
+#endif
+
 namespace dg {
 
 // First statement of every kernel that is launched with programmatic stream
@@ -375,26 +382,34 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
 // multiplied through by the density bound, with a 1e-5 margin relative to eabs >=
 // |E|, which covers the FP32 rounding of the inputs and of the test. The products
 // rho E and m^2 leave the range of binary32 in units as common as g / cm^3 (and 0
-// >= 0 would hold), so the test runs on rho, E and m scaled by powers of two 2^a,
-// 2^b and 2^((a + b) / 2) that bring rlo and eabs near 1: where the plain products
-// are in range the outcome is the same, bit for bit. Bounds below 2^-103 or
-// above 2^125, zeros, infinities and NaNs fail: the caller's next, FP64 test decides.
+// >= 0 would hold): where the margin itself is not well inside it, the test is made
+// on rho, E and m scaled by powers of two 2^a, 2^b and 2^((a + b) / 2) that bring rlo
+// and eabs near 1. Bounds below 2^-103 or above 2^125, zeros, infinities and
+// NaNs then fail: the caller's next, FP64 test decides.
 __device__ __forceinline__ bool pressure_clear_f32(float rlo, float elo, float eabs, const float (&mh)[3], float gm1,
                                                    float ep) {
-  // biased exponents (a set sign makes them large), their sum made even
-  const int xr = (int)(__float_as_uint(rlo) >> 23), x4 = (int)(__float_as_uint(eabs) >> 23);
-  if ((unsigned)(xr - 24) > 228u || (unsigned)(x4 - 24) > 228u) return false;
-  const int xe = x4 + ((xr + x4) & 1);
-  const float sr = __uint_as_float((unsigned)(254 - xr) << 23), se = __uint_as_float((unsigned)(254 - xe) << 23);
-  const float sm = __uint_as_float((unsigned)(254 - (xr + xe) / 2) << 23);
   float k2 = 0.f;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) k2 = fmaf(mh[a] * sm, mh[a] * sm, k2);
+  for (int a = 0; a < 3; ++a) k2 = fmaf(mh[a], mh[a], k2);
   k2 *= 0.5f;
-  const float r = rlo * sr;
-  const float lhs = gm1 * fmaf(elo * se, r, -k2);
-  const float rhs = fmaf(ep * se, r, 1e-5f * gm1 * fmaf(eabs * se, r, k2));
-  return lhs >= rhs;
+  float mg = 1e-5f * gm1 * fmaf(eabs, rlo, k2);
+  if (!(mg >= 1e-30f && mg <= 1e30f)) {
+    // biased exponents (a set sign makes them large), their sum made even
+    const int xr = (int)(__float_as_uint(rlo) >> 23), x4 = (int)(__float_as_uint(eabs) >> 23);
+    if ((unsigned)(xr - 24) > 228u || (unsigned)(x4 - 24) > 228u) return false;
+    const int xe = x4 + ((xr + x4) & 1);
+    const float sr = __uint_as_float((unsigned)(254 - xr) << 23), se = __uint_as_float((unsigned)(254 - xe) << 23);
+    const float sm = __uint_as_float((unsigned)(254 - (xr + xe) / 2) << 23);
+    rlo *= sr;
+    elo *= se;
+    ep *= se;
+    k2 = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) k2 = fmaf(mh[a] * sm, mh[a] * sm, k2);
+    k2 *= 0.5f;
+    mg = 1e-5f * gm1 * fmaf(eabs * se, rlo, k2);
+  }
+  return gm1 * fmaf(elo, rlo, -k2) >= fmaf(ep, rlo, mg);
 }
 
 // Sufficient limiter screen in FP32 from the cell means m and the excursion

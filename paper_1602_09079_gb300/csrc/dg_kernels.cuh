@@ -2151,10 +2151,45 @@ struct ResetSF {
   static constexpr int ROW = ((ROWW / 4) % 2 == 1 ? ROWW : ROWW + 4) * 4 / (int)sizeof(T);
   // dynamic shared memory: point values [4][C][ROW] and E [C][ROW]
   static constexpr size_t smem() { return (size_t)5 * C * ROW * sizeof(T); }
+  // CTAs per SM the register budget is sized for: what the kernel takes without
+  // reset_screen, which runs for few cells
+  static constexpr int MINB = sizeof(T) == 4 ? (K <= 2 ? 16 : 9) : (K <= 1 ? 10 : K == 2 ? 8 : 4);
 };
 
+// The FP64 test of a reset cell that the FP32 screen does not clear, on FP64 sums
+// (mixed: on the FP32 sums sA, widened). m, sa: means and sums of rho and the momenta,
+// en: energy modes (all 32 = C apart), y: the cell's coefficients. Not inlined and within
+// the kernel's own registers (MINB), which it would otherwise raise from 30 to 56:
+// reset and limiter at 100 x 90 x 84, degree 1, mixed, 73 us instead of 59 (57 without it).
 template <int K, typename T>
-__global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel(
+__device__ DG_NOINLINE bool reset_screen(const double* m, const double* sa, const double* en, const double* y,
+                                         long long nc, const T* __restrict__ tab, int vol, double gamma,
+                                         double eps_r, double eps_p) {
+  using TB = Tab<K>;
+  constexpr int C = ResetSF<K, T>::C, N = TB::N;
+  const int lmax = vol ? TB::LMAXV : TB::LMAX;
+  double md[5], ad[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    md[i] = i < 4 ? m[i * C] : en[0];
+    if constexpr (sizeof(T) == 8) {
+      ad[i] = 0.0;
+#pragma unroll 1
+      for (int l = 1; l < N; ++l) ad[i] += fabs(i < 4 ? y[(size_t)(i * N + l) * nc] : en[l * C]) * __ldg(tab + lmax + l);
+    } else if (i < 4) {
+      ad[i] = sa[i * C];
+    } else {
+      float se = 0.f;
+#pragma unroll 1
+      for (int l = 1; l < N; ++l) se += fabsf(f64_to_f32(en[l * C])) * c_tab32[lmax + l];
+      ad[i] = (double)se * (1.0 + 1e-5);
+    }
+  }
+  return limiter_screen<K>(md, ad, true, gamma, eps_r, eps_p);
+}
+
+template <int K, typename T>
+__global__ void __launch_bounds__(ResetSF<K, T>::THREADS, ResetSF<K, T>::MINB) energy_reset_sf_kernel(
     double* __restrict__ y, const T* __restrict__ tab, Geo g, ResetConsts<T> rc, double* __restrict__ part,
     int* __restrict__ list, Ctrl* ctrl, float* __restrict__ yf) {
   stream_wait();
@@ -2465,32 +2500,9 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS) energy_reset_sf_kernel
     }
     m[4] = f64_to_f32_q(sEn[c]);
     a[4] = sf * (1.f + 1e-5f);
-    bool queue = !fin || !screen_f32(m, a, (float)(g.gamma - 1.0), (float)g.eps_rho, (float)g.eps_p);
-    if (queue && fin) {
-      // the FP64 test decides, on FP64 sums (mixed: on the FP32 sums, widened)
-      double md[5], ad[5];
-#pragma unroll
-      for (int i = 0; i < 5; ++i) {
-        md[i] = i < 4 ? sM[i * C + c] : sEn[c];
-        if constexpr (sizeof(T) == 8) {
-          ad[i] = 0.0;
-#pragma unroll 1
-          for (int l = 1; l < N; ++l)
-            ad[i] += fabs(i < 4 ? y[(size_t)(i * N + l) * nc + cell] : sEn[l * C + c]) *
-                     __ldg(tab + (g.lim_vol ? TB::LMAXV : TB::LMAX) + l);
-        } else if (i < 4) {
-          ad[i] = sA[i * C + c];
-        } else {
-          float se = 0.f;
-#pragma unroll 1
-          for (int l = 1; l < N; ++l)
-            se += fabsf(f64_to_f32(sEn[l * C + c])) * c_tab32[(g.lim_vol ? TB::LMAXV : TB::LMAX) + l];
-          ad[i] = (double)se * (1.0 + 1e-5);
-        }
-      }
-      queue = !limiter_screen<K>(md, ad, true, g.gamma, g.eps_rho, g.eps_p);
-    }
-    if (queue) {
+    if (!fin || (!screen_f32(m, a, (float)(g.gamma - 1.0), (float)g.eps_rho, (float)g.eps_p) &&
+                 !reset_screen<K, T>(sM + c, sA + c, sEn + c, y + cell, nc, tab, g.lim_vol, g.gamma, g.eps_rho,
+                                     g.eps_p))) {
       const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
       list[slot] = (int)cell;
     }
