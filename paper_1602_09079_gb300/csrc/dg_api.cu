@@ -883,9 +883,6 @@ int dg_cfl_dt(dg_ctx* c, double courant, double* dt_out) {
   DG_TRY(need_bound(c));
   if (!dt_out || !(courant > 0.0)) return DG_ERR_ARG;
   DG_TRY(set_device(c));
-  // cleared by every call: nothing is left over from a reduction that was not
-  // launched, or from another context that uses this scratch in turn
-  DG_CUDA(cudaMemsetAsync(&c->ctrl->cfl_max_bits, 0, sizeof(unsigned long long), c->stream));
   DG_TRY(launch(c, KC_CFL, [&] { return c->fn.cfl(c->y, c->geo, c->ctrl, c->stream); }));
   Ctrl h{};
   int st = sync_and_check(c, &h);

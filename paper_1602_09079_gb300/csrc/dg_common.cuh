@@ -24,6 +24,13 @@ __device__ __forceinline__ void stream_wait() {
 #endif
 }
 
+// orders this thread's writes before its later ones for the whole device
+__device__ __forceinline__ void device_fence() {
+#ifdef __CUDA_ARCH__
+  __threadfence();
+#endif
+}
+
 // ------------------------------------------------------------- sizes
 __host__ __device__ constexpr int nmodes(int k) { return (k + 1) * (k + 2) * (k + 3) / 6; }
 __host__ __device__ constexpr int gll_m(int k) { return k <= 1 ? 2 : 3; }
@@ -142,7 +149,7 @@ enum : unsigned {
 // kernels and, before the fused stages and the reset, on the stream, and the
 // limiter's last pass clears it for the next stage.
 struct Ctrl {
-  unsigned long long cfl_max_bits;  // max over cells of the wave-speed sum (bits of a double >= 0)
+  unsigned long long cfl_max_bits;  // max over cells of the wave-speed sum (bits of a double >= 0): the result
   unsigned int err;                 // sticky ERRB_* bits
   unsigned int n_flag;              // cells queued for the full limiter
   unsigned long long n_limited;     // limiter count
@@ -150,6 +157,8 @@ struct Ctrl {
   unsigned int n_deep;              // queued cells the FP32 point screen does not clear
   unsigned long long n_queued_total;  // cells that failed the limiter screen (all stages)
   unsigned long long n_full_total;    // cells that went through the full limiter
+  unsigned long long cfl_running;     // of the reduction under way; 0 between the calls, like
+  unsigned int cfl_blocks;            // the number of its blocks that are done
   double sums[8];                     // results of the host-facing sums, read back with the error word
 };
 

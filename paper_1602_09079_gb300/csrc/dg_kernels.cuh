@@ -2105,8 +2105,18 @@ __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const double* __restri
       if (u > v) v = u;
     }
     if (threadIdx.x == 0) {
-      atomicMax(&ctrl->cfl_max_bits, v);
       if (s_err) atomicOr(&ctrl->err, s_err);
+      // the block that ends last hands the maximum over and leaves 0 for the next
+      // reduction, so that no call depends on another one having run (a memset
+      // before the kernel: 5 us of a host-bound loop on small meshes)
+      atomicMax(&ctrl->cfl_running, v);
+      device_fence();
+      if (atomicAdd(&ctrl->cfl_blocks, 1u) == gridDim.x - 1) {
+        device_fence();
+        ctrl->cfl_max_bits = atomicMax(&ctrl->cfl_running, 0ull);
+        ctrl->cfl_running = 0ull;
+        ctrl->cfl_blocks = 0u;
+      }
     }
   }
 }

@@ -42,7 +42,7 @@ struct Launchers {
   // screen[c] = 1 if cell c fails the limiter screen
   cudaError_t (*screen)(const double* y, uint8_t* screen, const Geo& g, cudaStream_t s);
   cudaError_t (*limit)(double* y, int8_t* flags, const Geo& g, Ctrl* ctrl, cudaStream_t s);
-  // into ctrl->cfl_max_bits (0 on entry)
+  // into ctrl->cfl_max_bits
   cudaError_t (*cfl)(const double* y, const Geo& g, Ctrl* ctrl, cudaStream_t s);
   // returns the number of partial sums written to part; cells failing the
   // limiter screen afterwards are queued in list / ctrl->n_flag (0 on entry)
