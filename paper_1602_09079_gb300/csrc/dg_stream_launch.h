@@ -21,7 +21,11 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t
   at.val.programmaticStreamSerializationAllowed = 1;
   c.attrs = &at;
   c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+  // the caller gets the error: not left for the next cudaGetLastError, here or in
+  // another library, to report as its own
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
 }
 
 }  // namespace dg
