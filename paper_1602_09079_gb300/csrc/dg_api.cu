@@ -344,6 +344,7 @@ struct dg_ctx {
   Ctrl* ctrl = nullptr;
   double* part = nullptr;
   double* modes_dev = nullptr;
+  bool queue_open = false;  // a failed call could not empty the limiter's queue (QueueUse)
   double* ybuf = nullptr;
   int* list = nullptr;
   int* list2 = nullptr;
@@ -444,13 +445,34 @@ int sync_and_check(dg_ctx* c, Ctrl* host_copy) {
   return err_to_status(h.err);
 }
 
-// Empties the limiter's queue: the first thing in a call that queues cells, whatever
-// an earlier call (of this context, or of another one on the same scratch) has left
-// there. Between the stages of a call the limiter's last pass leaves it empty; the
-// unfused stages' face kernels empty it themselves.
-int empty_queue(dg_ctx* c) {
-  return cuda_ok(cudaMemsetAsync(&c->ctrl->n_flag, 0, sizeof(unsigned), c->stream));
-}
+// Held by a call that queues cells for the limiter. The limiter's last pass leaves
+// the queue empty; a call that fails in between empties it before it returns, so
+// that neither this context's next call nor another one's on the same scratch finds
+// cells there. (A memset before every fused step and reset would do, but costs a
+// reset on 8^3 11 us.) Where that memset fails too, the next call repeats it first.
+class QueueUse {
+ public:
+  explicit QueueUse(dg_ctx* c) : c_(c) {}
+  ~QueueUse() {
+    if (!done_) c_->queue_open = !clear();
+  }
+  int begin() {
+    if (!c_->queue_open) return DG_OK;
+    if (!clear()) return DG_ERR_CUDA;
+    c_->queue_open = false;
+    return DG_OK;
+  }
+  void done() { done_ = true; }
+
+ private:
+  bool clear() {
+    if (cudaMemsetAsync(&c_->ctrl->n_flag, 0, sizeof(unsigned), c_->stream) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    return false;
+  }
+  dg_ctx* c_;
+  bool done_ = false;
+};
 
 int set_device(const dg_ctx* c) { return cuda_ok(cudaSetDevice(c->device)); }
 
@@ -540,6 +562,8 @@ int fused_step(dg_ctx* c, double dt, bool force) {
   const double a0[3] = {0.0, 0.75, 1.0 / 3.0};
   const double b0[3] = {1.0, 0.25, 2.0 / 3.0};
   const double* ys = c->y;
+  QueueUse queue(c);
+  DG_TRY(queue.begin());
   for (int s = 0; s < 3; ++s) {
     double* out = s == 0 ? c->ybuf : (s == 1 ? c->ybuf2 : c->y);
     FusedArgs a{};
@@ -557,7 +581,6 @@ int fused_step(dg_ctx* c, double dt, bool force) {
     a.b0_d = b0[s];
     a.y0 = c->y;
     a.stage = s + 1;
-    if (s == 0) DG_TRY(empty_queue(c));
     DG_TRY(launch(c, KC_VOLUME, [&] { return c->fz.run(force, c->flux, c->geo, a, c->stream); }));
     float* yf = s == 2 ? c->yf : nullptr;
     const double* y0 = s < 2 ? c->y : nullptr;
@@ -580,6 +603,7 @@ int fused_step(dg_ctx* c, double dt, bool force) {
     }
     ys = out;
   }
+  queue.done();
   c->limited = true;
   c->shadow_valid = true;
   return DG_OK;
@@ -678,6 +702,7 @@ int dg_bind(dg_ctx* c, double* y_dev, void* scratch_dev, size_t scratch_bytes, v
   c->ctrl = reinterpret_cast<Ctrl*>(c->scratch + L.ctrl);
   c->part = reinterpret_cast<double*>(c->scratch + L.part);
   c->modes_dev = reinterpret_cast<double*>(c->scratch + L.modes);
+  c->queue_open = false;
   c->ybuf = reinterpret_cast<double*>(c->scratch + L.ybuf);
   c->list = reinterpret_cast<int*>(c->scratch + L.list);
   c->list2 = reinterpret_cast<int*>(c->scratch + L.list2);
@@ -831,6 +856,7 @@ int dg_step(dg_ctx* c, double dt) {
   const double a0[3] = {0.0, 0.75, 1.0 / 3.0};
   const double b0[3] = {1.0, 0.25, 2.0 / 3.0};
   const double* ys = c->y;
+  QueueUse queue(c);
   for (int s = 0; s < 3; ++s) {
     double* out = s < 2 ? c->ybuf : c->y;
     DG_TRY(launch(c, KC_FACE, [&] { return c->fn.face(c->prec, c->flux, ys, yf, c->fh, c->geo, c->ctrl, c->stream); }));
@@ -858,6 +884,7 @@ int dg_step(dg_ctx* c, double dt) {
     }
     ys = out;
   }
+  queue.done();
   c->limited = true;
   c->shadow_valid = shadow;
   return DG_OK;
@@ -963,7 +990,8 @@ int dg_energy_reset(dg_ctx* c, double c_iso, double rho0, double* dissipated) {
   // keep the FP32 shadow current if it is (energy rows and limited cells)
   float* yf = (uses_shadow(c) && c->shadow_valid) ? c->yf : nullptr;
   if (!yf) c->shadow_valid = false;
-  DG_TRY(empty_queue(c));
+  QueueUse queue(c);
+  DG_TRY(queue.begin());
   DG_TRY(launch(c, KC_RESET, [&] {
     return c->fn.energy_reset(c->prec, c->y, c->geo, c2g, 1.0 / rho0, c->part, &n_part, c->list, c->ctrl, yf,
                               c->stream);
@@ -974,6 +1002,7 @@ int dg_energy_reset(dg_ctx* c, double c_iso, double rho0, double* dissipated) {
     return c->fn.limit_list(c->y, c->list, &c->ctrl->n_flag, c->geo, c->ctrl, 0, yf, nullptr, nullptr, c->list2,
                                 c->stream);
   }, 2));
+  queue.done();
   c->limited = true;
   if (dissipated) {
     const double vol = c->geo.dx[0] * c->geo.dx[1] * c->geo.dx[2];

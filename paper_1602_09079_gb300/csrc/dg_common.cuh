@@ -143,11 +143,11 @@ enum : unsigned {
   ERRB_NEWTON = 4u,
 };
 
-// Control block at the start of the scratch buffer. No call relies on what another
-// one leaves in the queue counters: every stage (and the energy reset) clears n_deep
-// before its cells are queued; n_flag is cleared by the unfused stages' face
-// kernels and, before the fused stages and the reset, on the stream, and the
-// limiter's last pass clears it for the next stage.
+// Control block at the start of the scratch buffer. The queue counters: every stage
+// (and the energy reset) clears n_deep before its cells are queued; n_flag is 0
+// between the stages and between the calls (the limiter's last pass clears it, and
+// a call that fails before that does on the stream); the unfused stages' face kernels
+// clear it in any case.
 struct Ctrl {
   unsigned long long cfl_max_bits;  // max over cells of the wave-speed sum (bits of a double >= 0): the result
   unsigned int err;                 // sticky ERRB_* bits

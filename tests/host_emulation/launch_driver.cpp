@@ -13,8 +13,8 @@
 //       segment
 //   launch_driver step nx ny nz prec gamma eps_rho eps_p lim_vol in.bin out.bin dt n_modes modes.bin c_iso rho0 seg
 //       one dg_step in the unit box, then (c_iso > 0) dg_energy_reset. The queue's
-//       counter starts with something else's value and is cleared on the stream only
-//       where the C ABI does that (before the fused stages and the reset)
+//       counter is as the kernels leave it; before the unfused stages, whose face
+//       kernels clear it, it starts with another value
 //
 // States in the state layout [5][N][n_cells], FP64. Prints "err=<device error
 // word>" and what else a command says.
@@ -219,11 +219,10 @@ static void step_launch(Setup& S, std::vector<double>& y, double dt, const std::
   std::vector<int> list(nc, -1), deep(nc, -1);
   const double a0[3] = {0.0, 0.75, 1.0 / 3.0}, b0[3] = {1.0, 0.25, 2.0 / 3.0};
   const double* ys = y.data();
-  S.ctrl.n_flag = 3;
+  S.ctrl.n_flag = sizeof(T) == 4 && K >= 1 ? 0 : 3;
   for (int s = 0; s < 3; ++s) {
 #if DG_K >= 1
     if constexpr (sizeof(T) == 4) {
-      if (s == 0) S.ctrl.n_flag = 0;
       launch_fused_setup(S);
       double* out = s == 0 ? ybuf.data() : (s == 1 ? ybuf2.data() : y.data());
       FusedArgs a{};
@@ -257,7 +256,6 @@ static void step_launch(Setup& S, std::vector<double>& y, double dt, const std::
   }
   double diss = 0.0;
   if (c_iso > 0.0) {
-    S.ctrl.n_flag = 0;
     const unsigned nbr = grid1(nc, 32);
     std::vector<double> part(nbr, 0.0);
     ResetConsts<T> rc;

@@ -2,7 +2,10 @@
 objects linked against a fake runtime on host memory (tests/host_emulation/
 fake_cudart.cpp; kernels do not run): the error is returned and not left behind as
 the thread's last error, where the next launch, of this library or of another one,
-would report it as its own."""
+would report it as its own. A step or a reset that fails after cells may have been
+queued for the limiter leaves the queue's count at 0, for every launch that can
+fail; if even that memset is refused, the next call that relies on the count starts
+with it. A CFL reduction that was not launched leaves nothing behind."""
 import ctypes as C
 import os
 import shutil
@@ -14,6 +17,7 @@ import paper_1602_09079_gb300 as dg
 from paper_1602_09079_gb300 import _build
 
 EMU = os.path.join(os.path.dirname(os.path.abspath(__file__)), "host_emulation")
+N_FLAG = 3  # 32-bit word of the control block at the start of the scratch
 
 
 @pytest.fixture(scope="module")
@@ -80,3 +84,43 @@ def test_error_is_not_left_behind(lib, order, mixed, call):
         assert run() == dg.DG_ERR_CUDA
         assert lib.fake_pending_error() == 0
         assert calls(b)["limit"]() == 0
+
+
+@pytest.mark.parametrize("order", [1, 2, 3, 4])
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("call", ["step", "reset"])
+def test_queue_is_empty_after_a_failed_call(lib, order, mixed, call):
+    b = Bound(lib, order, mixed)
+    run = calls(b)[call]
+    assert run() == 0  # the first step limits its input
+    lib.fake_fail(-1, 0)
+    assert run() == 0
+    n = lib.fake_launches()
+    assert n >= (6 if call == "step" else 3)
+    for j in range(n):
+        b.words[N_FLAG] = 7  # what that launch would have queued
+        lib.fake_fail(j, 0)
+        assert run() == dg.DG_ERR_CUDA
+        assert b.words[N_FLAG] == 0, j
+        # the same where the memset is refused too: the next call begins with it
+        b.words[N_FLAG] = 7
+        lib.fake_fail(j, 1)
+        assert run() == dg.DG_ERR_CUDA
+        lib.fake_fail(-1, 0)
+        assert b.lib.dg_energy_reset(b.ctx, 1.0, 1.0, None) == 0
+        assert b.words[N_FLAG] == 0 and lib.fake_memsets() == 1
+
+
+@pytest.mark.parametrize("order", [1, 3])
+def test_cfl_reduction_that_was_not_launched(lib, order):
+    """With kernels that do not run, dg_cfl_dt reads the result that the control
+    block holds: the same word whatever calls failed before."""
+    b = Bound(lib, order, False)
+    result = C.c_double.from_address(b.scratch)
+    dt = C.c_double()
+    for fail in (-1, 0, -1, 0, 0, -1):
+        result.value = 2.0
+        lib.fake_fail(fail, 0)
+        st = b.lib.dg_cfl_dt(b.ctx, 0.3, C.byref(dt))
+        assert st == (0 if fail < 0 else dg.DG_ERR_CUDA)
+        assert result.value == 2.0
