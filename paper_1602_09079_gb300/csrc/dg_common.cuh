@@ -689,11 +689,13 @@ __device__ __forceinline__ double rsqrt64(double x) {
   const unsigned odd = (unsigned)(bx - 1023) & 1u;
   const int half = (bx - 1023 - (int)odd) >> 1;
   const unsigned f = ((127u + odd) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const unsigned y0 = (unsigned)(rsqrt_fast(__uint_as_float(f)) * 0x1p30f);
+  // in units of 2^-24: below 0.5 (significands just under 4) the approximation has a
+  // bit more, which the residual could not see
+  const unsigned y0 = (unsigned)(rsqrt_fast(__uint_as_float(f)) * 0x1p30f) & ~63u;
   // significand in [1, 4), 54 bits
   const unsigned long long m = (((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << odd;
   const unsigned a0 = (unsigned)m, a1 = (unsigned)(m >> 32);
-  const unsigned k = y0 >> 6;  // y0's 24 bits: units of 2^-24, exact
+  const unsigned k = y0 >> 6;
   const unsigned long long s = (unsigned long long)k * k;
   const unsigned s0 = (unsigned)s, s1 = (unsigned)(s >> 32);
   // 1 - m y0^2 in units of 2^-82, modulo 2^64
