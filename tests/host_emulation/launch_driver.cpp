@@ -16,6 +16,10 @@
 //       counter is as the kernels leave it; before the unfused stages, whose face
 //       kernels clear it, it starts with another value
 //
+//   launch_driver fft M in.bin out.bin
+//       shell sums of the M^3 real samples in in.bin by the library's own transform
+//       (M = 32 .. 1024 a power of two)
+//
 // States in the state layout [5][N][n_cells], FP64. Prints "err=<device error
 // word>" and what else a command says.
 #include <type_traits>
@@ -24,6 +28,18 @@
 #define main driver_main
 #include "driver.cpp"
 #undef main
+struct longlong2 {
+  long long x, y;
+};
+inline void sincospi(double x, double* s, double* c) {
+  *s = (double)sinl(3.14159265358979323846264338327950288L * x);
+  *c = (double)cosl(3.14159265358979323846264338327950288L * x);
+}
+namespace dg {
+namespace spec {
+#include "fft_kernels.inc"
+}  // namespace spec
+}  // namespace dg
 
 // the launcher's grid of a kernel over a queue (limit_grid)
 static unsigned queue_grid(long long nc, int per, unsigned most) {
@@ -291,8 +307,39 @@ static int run_step_launch(int argc, char** argv) {
   return write_file(argv[11], y.data(), y.size()) ? 0 : 3;
 }
 
+static int run_fft(int argc, char** argv) {
+  if (argc != 5) return 2;
+  using namespace spec;
+  const int M = std::atoi(argv[2]);
+  if (!own_fft(M)) return 2;
+  // sizes and launches of own_spectrum
+  const int nb = (int)std::floor(std::sqrt(3.0) * M / 2.0) + 2, lines = kFftPoints / M;
+  const int copies = nb * 64 <= 48 * 1024 ? 8 : 1;
+  int logm = 0;
+  while ((1 << logm) < M) ++logm;
+  const size_t rows = sizeof(Cx) * (size_t)lines * (M + 1) + 8 * (size_t)lines;
+  const size_t cols = sizeof(Cx) * (size_t)kFftPoints + 8 * (size_t)lines;
+  const size_t colz = cols + sizeof(double) * (size_t)nb * copies;
+  std::vector<double> real((size_t)M * M * M), bins(nb, 0.0);
+  if (!read_file(argv[3], real.data(), real.size())) return 3;
+  std::vector<double2> cplx((size_t)M * M * (M / 2), double2{std::nan(""), std::nan("")});
+  std::vector<longlong2> tw(M);
+  const unsigned tiles = (unsigned)((long long)M * M / 2 / lines);
+  emu::launch((M + 255) / 256, 256, 0, [&] { twiddle_kernel(M, tw.data()); });
+  emu::launch(tiles, 256, rows, [&] { fft_rows_kernel(real.data(), cplx.data(), M, logm, tw.data()); });
+  emu::launch(tiles, 256, cols, [&] { fft_lines_kernel<false>(cplx.data(), M, logm, tw.data(), nb, 1, nullptr); });
+  emu::launch(std::min(tiles, 152u * 2), 256, colz,
+              [&] { fft_lines_kernel<true>(cplx.data(), M, logm, tw.data(), nb, copies, bins.data()); });
+  emu::launch((unsigned)(((long long)M * M + 255) / 256), 256, 0,
+              [&] { fft_packed_bins_kernel(cplx.data(), M, nb, bins.data()); });
+  if (!write_file(argv[4], bins.data(), bins.size())) return 3;
+  std::printf("bins=%d\n", nb);
+  return 0;
+}
+
 int main(int argc, char** argv) {
   if (argc < 2) return 2;
+  if (std::strcmp(argv[1], "fft") == 0) return run_fft(argc, argv);
   if (std::strcmp(argv[1], "queue") == 0) return run_queue(argc, argv);
   if (std::strcmp(argv[1], "limit") == 0) return run_limit(argc, argv);
   if (std::strcmp(argv[1], "rhs") == 0) return run_rhs_launch(argc, argv);
