@@ -1162,8 +1162,9 @@ struct VolSF<K, double> {
   static constexpr int A = 18 * Q3 * C, B = SCREEN + ((Q + 1) * 5 * C + 1) / 2, END = A > B ? A : B;
   static constexpr size_t smem() { return sizeof(double) * END; }
   // CTAs per SM the register budget is sized for (128^3, degree 2: 5.5 ms with 3, 7.1
-  // with 2; degree 3 has no shared memory for a third)
-  static constexpr int MINB = K <= 2 ? 3 : 2;
+  // with 2; 64^3, degree 1: 0.219 ms with 4, 0.215 with 3, driven 0.271 and 0.305;
+  // degree 3 has no shared memory for a third)
+  static constexpr int MINB = K == 1 ? 4 : (K == 2 ? 3 : 2);
   // directions whose faces one slice's threads take
   static constexpr int NF = (2 + Q) / Q;
 };
