@@ -90,7 +90,11 @@ int dg_sizes(const dg_ctx* ctx, int features, size_t* state_len, size_t* scratch
  * legacy default stream). y_dev: state layout, 5 N n_cells doubles, 8-byte
  * aligned; scratch_dev: at least dg_sizes(ctx, 0, ...) bytes, 256-byte
  * aligned; a scratch of dg_sizes(ctx, DG_FEATURE_FORCING, ...) bytes enables
- * dg_set_forcing. Errors: DG_ERR_ARG (NULL, misaligned, too small). */
+ * dg_set_forcing. Contexts may use one scratch in turn, on one stream, in FP64
+ * and without driving: no call relies on what another one has left there, but for
+ * the sticky error word and the limiter counts, which the scratch holds. (The mixed
+ * path keeps the state's FP32 copy in it, the driving its field, so these need a
+ * scratch of their own.) Errors: DG_ERR_ARG (NULL, misaligned, too small). */
 int dg_bind(dg_ctx* ctx, double* y_dev, void* scratch_dev, size_t scratch_bytes, void* cuda_stream);
 
 /* Copy a canonical-layout state (host if is_device == 0, else device) into

@@ -2,9 +2,10 @@
 // E_w(k) is the shell average of |w_hat(k)|^2 scaled so that its integral
 // over k equals the mean square of w. Here the velocity of the state
 // polynomial is sampled at sub^3 points per cell (cell-centred sub-cells),
-// each component is transformed by a 3D real-to-complex FFT (cuFFT, on a
-// caller-provided work area), and the power of every wave vector n is added
-// to the shell round(|n|).
+// each component is transformed by a 3D real-to-complex FFT on a
+// caller-provided work area (own passes in fixed point for grids of 32 to 1024
+// points a side, a power of two; cuFFT for the others), and the power of every
+// wave vector n is added to the shell round(|n|).
 #include "dg_spectrum.h"
 
 #include <cufft.h>
