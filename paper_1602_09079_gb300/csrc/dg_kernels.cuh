@@ -105,30 +105,6 @@ __device__ __forceinline__ bool limiter_screen(const double* mean, const double*
   return plo >= eps_p + 1e-13 * gm1 * (fabs(mean[4]) + sabs[4] + kin);
 }
 
-// The same of a cell whose new coefficients w (rows nc apart) a thread reads back:
-// decides for the cells that an FP32 screen does not clear, so that the FP64
-// path's queue (dg_limiter_counts, the indicator's input) is decided in FP64
-template <int K>
-__device__ bool limiter_screen_of(const double* w, size_t nc, const double* __restrict__ lmax,
-                                               const Geo& g) {
-  constexpr int N = nmodes(K);
-  double m[5], a[5];
-  bool fin = true;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    m[i] = w[(size_t)(i * N) * nc];
-    fin &= finite64(m[i]);
-    a[i] = 0.0;
-#pragma unroll 1
-    for (int l = 1; l < N; ++l) {
-      const double v = w[(size_t)(i * N + l) * nc];
-      a[i] += fabs(v) * __ldg(lmax + l);
-      fin &= finite64(v);
-    }
-  }
-  return limiter_screen<K>(m, a, fin, g.gamma, g.eps_rho, g.eps_p);
-}
-
 // --------------------------------------------------------------- volume
 template <int K, typename T, int MODE, bool FORCE>
 __global__ void __launch_bounds__(kThreads) volume_kernel(const double* __restrict__ yin, const T* __restrict__ fh,
@@ -1653,10 +1629,16 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
   }
   if (MODE == MODE_RHS) return;
   // limiter screen of the next stage's input: FP32 (sufficient) for all cells,
-  // FP64 for those it does not clear; what fails both is queued for the full limiter
+  // FP64 for those it does not clear, so that dg_limiter_counts and the
+  // indicator's input are decided in FP64; what fails both is queued for the full
+  // limiter. The FP64 sums are taken by the threads that hold the modes: one thread
+  // reading 5 N coefficients one after the other took 10 us.
   sScr[(qz * 5 + i) * C + c] = sab * (1.f + 1e-5f);
   __syncthreads();
-  if (tid < C && live) {
+  int* sTest = reinterpret_cast<int*>(smem_raw);  // [C]; the sums before are done with
+  double* sSum = sm64 + C;                        // [Q][5][C]
+  bool test = false;
+  if (tid < C) {
     float m[5], s[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
@@ -1665,8 +1647,33 @@ __global__ void __launch_bounds__(kThreads, VolSF<K, double>::MINB)
 #pragma unroll
       for (int z = 0; z < Q; ++z) s[v] += sScr[(z * 5 + v) * C + tid];
     }
-    if (!screen_f32(m, s, (float)gm1, (float)g.eps_rho, (float)g.eps_p) &&
-        !limiter_screen_of<K>(st.out + cell, nc, tab64 + (g.lim_vol ? TB::LMAXV : TB::LMAX), g)) {
+    test = live && !screen_f32(m, s, (float)gm1, (float)g.eps_rho, (float)g.eps_p);
+    sTest[tid] = test;
+  }
+  __syncthreads();
+  if (sTest[c]) {
+    double s = 0.0;
+#pragma unroll
+    for (int j = 0; j * Q < N; ++j) {
+      const int l = qz + j * Q;
+      if (l > 0 && l < N)
+        s += fabs(st.out[(size_t)(i * N + l) * nc + cell]) * __ldg(tab64 + (g.lim_vol ? TB::LMAXV : TB::LMAX) + l);
+    }
+    sSum[(qz * 5 + i) * C + c] = s;
+  }
+  __syncthreads();
+  if (test) {
+    double m[5], s[5];
+    bool fin = true;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      m[v] = st.out[(size_t)(v * N) * nc + cell];
+      s[v] = 0.0;
+#pragma unroll
+      for (int z = 0; z < Q; ++z) s[v] += sSum[(z * 5 + v) * C + tid];
+      fin &= finite64(m[v]) && finite64(s[v]);
+    }
+    if (!limiter_screen<K>(m, s, fin, g.gamma, g.eps_rho, g.eps_p)) {
       const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
       st.list[slot] = (int)cell;
     }
@@ -2167,34 +2174,34 @@ struct ResetSF {
   static constexpr int MINB = sizeof(T) == 4 ? (K <= 2 ? 16 : 9) : (K <= 1 ? 10 : K == 2 ? 8 : 4);
 };
 
-// The FP64 test of a reset cell that the FP32 screen does not clear, on FP64 sums
-// (mixed: on the FP32 sums sA, widened). m, sa: means and sums of rho and the momenta,
-// en: energy modes (all 32 = C apart), y: the cell's coefficients. Not inlined and within
-// the kernel's own registers (MINB), which it would otherwise raise from 30 to 56:
-// reset and limiter at 100 x 90 x 84, degree 1, mixed, 73 us instead of 59 (57 without it).
+// The FP64 test of a reset cell that the FP32 screen does not clear. m, sa: means and
+// sums of rho and the momenta, en: energy modes (all 32 = C apart), whose sum is taken
+// in T's precision (FP32: widened). Not inlined and within the kernel's own
+// registers (MINB), which it would otherwise raise from 30 to 56: reset and limiter at
+// 100 x 90 x 84, degree 1, mixed, 73 us instead of 59 (57 without it).
 template <int K, typename T>
-__device__ DG_NOINLINE bool reset_screen(const double* m, const double* sa, const double* en, const double* y,
-                                         long long nc, const T* __restrict__ tab, int vol, double gamma,
-                                         double eps_r, double eps_p) {
+__device__ DG_NOINLINE bool reset_screen(const double* m, const double* sa, const double* en,
+                                         const T* __restrict__ tab, int vol, double gamma, double eps_r,
+                                         double eps_p) {
   using TB = Tab<K>;
   constexpr int C = ResetSF<K, T>::C, N = TB::N;
   const int lmax = vol ? TB::LMAXV : TB::LMAX;
   double md[5], ad[5];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    md[i] = i < 4 ? m[i * C] : en[0];
-    if constexpr (sizeof(T) == 8) {
-      ad[i] = 0.0;
+  for (int i = 0; i < 4; ++i) {
+    md[i] = m[i * C];
+    ad[i] = sa[i * C];
+  }
+  md[4] = en[0];
+  if constexpr (sizeof(T) == 8) {
+    ad[4] = 0.0;
 #pragma unroll 1
-      for (int l = 1; l < N; ++l) ad[i] += fabs(i < 4 ? y[(size_t)(i * N + l) * nc] : en[l * C]) * __ldg(tab + lmax + l);
-    } else if (i < 4) {
-      ad[i] = sa[i * C];
-    } else {
-      float se = 0.f;
+    for (int l = 1; l < N; ++l) ad[4] += fabs(en[l * C]) * __ldg(tab + lmax + l);
+  } else {
+    float se = 0.f;
 #pragma unroll 1
-      for (int l = 1; l < N; ++l) se += fabsf(f64_to_f32(en[l * C])) * c_tab32[lmax + l];
-      ad[i] = (double)se * (1.0 + 1e-5);
-    }
+    for (int l = 1; l < N; ++l) se += fabsf(f64_to_f32(en[l * C])) * c_tab32[lmax + l];
+    ad[4] = (double)se * (1.0 + 1e-5);
   }
   return limiter_screen<K>(md, ad, true, gamma, eps_r, eps_p);
 }
@@ -2486,9 +2493,9 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS, ResetSF<K, T>::MINB) e
   __syncthreads();
   // ------------------------------- screen of the reset state, dissipation
   double diss = 0.0;
+  bool queue = false, test = false;
   if (tid < C && c0 + tid < nc) {
     const int c = tid;
-    const long long cell = c0 + c;
     bool fin = finite64(sEn[c]);
     float sf = 0.f;
 #pragma unroll
@@ -2511,13 +2518,10 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS, ResetSF<K, T>::MINB) e
     }
     m[4] = f64_to_f32_q(sEn[c]);
     a[4] = sf * (1.f + 1e-5f);
-    if (!fin || (!screen_f32(m, a, (float)(g.gamma - 1.0), (float)g.eps_rho, (float)g.eps_p) &&
-                 !reset_screen<K, T>(sM + c, sA + c, sEn + c, y + cell, nc, tab, g.lim_vol, g.gamma, g.eps_rho,
-                                     g.eps_p))) {
-      const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
-      list[slot] = (int)cell;
-    }
+    queue = !fin;
+    test = fin && !screen_f32(m, a, (float)(g.gamma - 1.0), (float)g.eps_rho, (float)g.eps_p);
   }
+  if (tid < C) sFin[tid] = test;
   // block sum of the dissipation: the C = 32 cells are warp 0's (fixed
   // shuffle order: deterministic)
   if (tid < 32) {
@@ -2532,6 +2536,26 @@ __global__ void __launch_bounds__(ResetSF<K, T>::THREADS, ResetSF<K, T>::MINB) e
       y[(size_t)(4 * N + l) * nc + cell] = sEn[l * C + c];
       if (yf) yf[(size_t)(4 * N + l) * nc + cell] = f64_to_f32(sEn[l * C + c]);
     }
+  }
+  // cells that the FP32 screen does not clear: FP64 sums of rho and the momenta (a
+  // warp per variable), then the FP64 test
+  if constexpr (sizeof(T) == 8) {
+    __syncthreads();
+    const int i = tid / C, c = tid % C;
+    if (sFin[c]) {
+      double sa = 0.0;
+#pragma unroll
+      for (int l = 1; l < N; ++l)
+        sa += fabs(y[(size_t)(i * N + l) * nc + c0 + c]) * __ldg(tab + (g.lim_vol ? TB::LMAXV : TB::LMAX) + l);
+      sA[i * C + c] = sa;
+    }
+    __syncthreads();
+  }
+  if (test)
+    queue = !reset_screen<K, T>(sM + tid, sA + tid, sEn + tid, tab, g.lim_vol, g.gamma, g.eps_rho, g.eps_p);
+  if (queue) {
+    const unsigned slot = atomicAdd(&ctrl->n_flag, 1u);
+    list[slot] = (int)(c0 + tid);
   }
 }
 
