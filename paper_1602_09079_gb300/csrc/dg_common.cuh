@@ -24,10 +24,15 @@ __device__ __forceinline__ void stream_wait() {
 #endif
 }
 
-// orders this thread's writes before its later ones for the whole device
-__device__ __forceinline__ void device_fence() {
+// adds 1 to a counter and returns the old value; this thread's earlier atomics are
+// visible to whoever sees the addition, and those of the earlier counts to this thread
+__device__ __forceinline__ unsigned count_done(unsigned* p) {
 #ifdef __CUDA_ARCH__
-  __threadfence();
+  unsigned r;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(r) : "l"(__cvta_generic_to_global(p)) : "memory");
+  return r;
+#else
+  return __atomic_fetch_add(p, 1u, __ATOMIC_ACQ_REL);
 #endif
 }
 
@@ -468,8 +473,7 @@ __device__ __forceinline__ Fx fx_split(long long r) { return {(int)(r >> 30), (i
 // the same with -2^29 <= l < 2^29, for |r| < 2^60.9: where many products go into
 // one sum, low limbs that are never negative would not cancel in its mid
 __device__ __forceinline__ Fx fx_split_signed(long long r) {
-  const int l = ((int)(r & 0x3fffffff) ^ 0x20000000) - 0x20000000;
-  return {(int)((r - l) >> 30), l};
+  return {(int)((r + 0x20000000) >> 30), (int)((unsigned)r << 2) >> 2};
 }
 __device__ __forceinline__ long long fx_join(Fx x) { return (long long)x.h * (1 << 30) + x.l; }
 __device__ __forceinline__ void fx_mad(FxAcc& a, Fx x, int ch, int cl) {
@@ -1036,16 +1040,18 @@ __device__ __forceinline__ double exp_add(double x, int de) {
 // powers of two 2^r, 2^e and 2^((r + e) / 2) that bring rho, E and the momenta near
 // 1. rho E and m^2 scale alike, so the screens decide as they would in binary32
 // of unlimited range. Means near the ends of the FP64 range (ok unset) are left
-// to the FP64 limiter.
+// to the FP64 limiter; between 2^-20 and 2^20 (plain) every product of the screens is in
+// range as it is, and they decide the same without the scaling.
 struct LimUnits {
   int r, m, e;
-  bool ok;
+  bool ok, plain;
   __device__ __forceinline__ LimUnits(double rho, double E) {
     const int br = bexp((unsigned)__double2hiint(rho)), be = bexp((unsigned)__double2hiint(E));
     ok = (unsigned)(br - 64) <= 1900u && (unsigned)(be - 64) <= 1900u;
     r = 1023 - br;
     e = 1023 - be - ((br + be) & 1);
     m = (r + e) / 2;
+    plain = (unsigned)(br - 1003) <= 39u && (unsigned)(be - 1003) <= 39u;
   }
   __device__ __forceinline__ int of(int i) const { return i == 0 ? r : (i == 4 ? e : m); }
 };
